@@ -17,10 +17,10 @@ OUT_DIR = os.path.join(HERE, "_lib")
 LIB = os.path.join(OUT_DIR, "liblbm.so")
 INCLUDE = os.path.join(os.path.dirname(HERE), "include")
 
-# (source, extra defines): step_inst.cu is built once per (lattice, precision)
-SOURCES = [("lbm_api.cu", []), ("lattice_table.cpp", []), ("lbm_slab.cpp", []), ("lbm_noalloc.cu", []),
-           ("lbm_pool.cu", [])] + [
-    ("step_inst.cu", [f"-DLBM_LAT={lat}", f"-DLBM_PREC={prec}"]) for lat in (0, 1) for prec in (0, 1, 2, 3)]
+# (source, extra defines): step_inst.cu is built once per (lattice, precision, part); the long ones first
+SOURCES = [("step_inst.cu", [f"-DLBM_LAT={lat}", f"-DLBM_PREC={prec}", f"-DLBM_PART={part}"])
+           for lat in (1, 0) for part in (1, 2, 0) for prec in (2, 3, 1, 0)] + [
+    ("lbm_api.cu", []), ("lattice_table.cpp", []), ("lbm_slab.cpp", []), ("lbm_noalloc.cu", []), ("lbm_pool.cu", [])]
 NVCC = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "--expt-relaxed-constexpr", "-Xcompiler", "-fPIC",
@@ -55,7 +55,7 @@ def build(force: bool = False, verbose: bool = False, extra_flags=None) -> str:
             sys.stderr.write(p.stdout + p.stderr)
         return obj
 
-    with ThreadPoolExecutor(max_workers=len(SOURCES)) as ex:
+    with ThreadPoolExecutor(max_workers=max(8, os.cpu_count() or 1)) as ex:
         objs = list(ex.map(compile_one, SOURCES))
     tmp = LIB + ".tmp"
     cmd = [NVCC, *ARCH, "-shared", "-o", tmp, *objs]

@@ -205,6 +205,77 @@ __device__ __forceinline__ void scale_gh(C& g, C& h, int grp, const Args<C>& a) 
 }
 
 // ---------------------------------------------------------------------------
+// read-only loads that stay where they are written: not merged with another of
+// the same address, not moved past one another
+__device__ __forceinline__ float ld_again(const float* p) {
+  float v;
+  asm volatile("ld.global.nc.f32 %0, [%1];" : "=f"(v) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ uint4 ld_again(const uint4* p) {
+  uint4 v;
+  asm volatile("ld.global.nc.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ double ld_again(const double* p) {
+  double v;
+  asm volatile("ld.global.nc.f64 %0, [%1];" : "=d"(v) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ unsigned ld_again(const unsigned* p) {
+  unsigned v;
+  asm volatile("ld.global.nc.b32 %0, [%1];" : "=r"(v) : "l"(p));
+  return v;
+}
+
+__device__ __forceinline__ float2 ld_again(const float2* p) {
+  float2 v;
+  asm volatile("ld.global.nc.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ uint2 ld_again(const uint2* p) {
+  uint2 v;
+  asm volatile("ld.global.nc.v2.b32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "l"(p));
+  return v;
+}
+
+// ---------------------------------------------------------------------------
+// two FP32 values in one 64-bit register; add, multiply and fma work on both
+// in one instruction, each rounded as the scalar one is
+// ---------------------------------------------------------------------------
+using f32x2 = unsigned long long;
+__device__ __forceinline__ f32x2 pack_f32x2(float a, float b) {
+  f32x2 v;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "f"(a), "f"(b));
+  return v;
+}
+__device__ __forceinline__ f32x2 both(float a) { return pack_f32x2(a, a); }
+__device__ __forceinline__ void unpack_f32x2(f32x2 v, float& a, float& b) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+}
+__device__ __forceinline__ f32x2 add_f32x2(f32x2 a, f32x2 b) {
+  f32x2 v;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(v) : "l"(a), "l"(b));
+  return v;
+}
+__device__ __forceinline__ f32x2 sub_f32x2(f32x2 a, f32x2 b) {
+  f32x2 v;
+  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(v) : "l"(a), "l"(b));
+  return v;
+}
+__device__ __forceinline__ f32x2 neg_f32x2(f32x2 a) { return a ^ 0x8000000080000000ull; }
+__device__ __forceinline__ f32x2 mul_f32x2(f32x2 a, f32x2 b) {
+  f32x2 v;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(v) : "l"(a), "l"(b));
+  return v;
+}
+__device__ __forceinline__ f32x2 fma_f32x2(f32x2 a, f32x2 b, f32x2 c) {
+  f32x2 v;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(v) : "l"(a), "l"(b), "l"(c));
+  return v;
+}
+
+// ---------------------------------------------------------------------------
 // equilibrium deviations (Eq. (18), regrouped by powers of s per group)
 //
 // With u2 = |u|^2, t = T - 1, x2 = |xi|^2 of the group:
@@ -1477,29 +1548,36 @@ __global__ void k_moments(const S* __restrict__ src, double* __restrict__ rho, d
   T[cell] = T0 + static_cast<double>(dT);
 }
 
-// deviations (dg_i, dh_i) of a cell in double for the FP64 reductions
-// (16-bit codec evaluated in FP32, as the step evaluates it)
-template <int Q, class S>
-__device__ __forceinline__ void decode_pair_d(const S* __restrict__ src, int i, long long ps, size_t cell, int grp,
-                                              const Args<float>& af, double& g, double& h) {
-  if constexpr (IsS16<S>::value) {
-    float gr, hr;
-    ld_gh<Q, S, float>(src, i, ps, cell, gr, hr);
-    g = static_cast<double>(gr * af.gref[grp]);
-    h = static_cast<double>(hr * af.hscale[grp]);
-  } else {
-    ld_gh<Q, S, double>(src, i, ps, cell, g, h);
-  }
-}
-
 // ---------------------------------------------------------------------------
 // FP64 conservation sums of the deviations: per-block partials, then one
 // fixed-order final pass; the host adds the reference totals N rho0 (mass)
 // and N rho0 (D + delta) T0 / 2 (energy)
+//
+// The totals are bound by the FP64 pipe (2 instructions per SM and clock)
+// long before HBM: a term-by-term FP64 sum takes about 5 FP64 instructions
+// per direction (185 per D2Q37 cell, plus a conversion per value), and HBM
+// delivers a cell's FP32 values every 26.  So FP32 and 16-bit storage sum on
+// the FP32 pipe first, without losing a bit of a term: every accumulator is
+// an unevaluated sum hi + lo, each addition to hi keeps its rounding error
+// (Knuth's two-sum) and adds it to lo.  There is one accumulator per
+// velocity group (for mass and kinetic energy), one for h, and one per axis
+// and |c_a| (momentum); after at most kTotalsRun cells of a thread they are
+// added up in FP64 with the factors c, |c|^2.  lo's own rounding is 2^-24 of
+// lo, at most (terms) 2^-48 of hi; against exact sums of the stored values
+// the totals are as near as the term-by-term FP64 sum's (2e-16 of the mass
+// and of the energy).  A run whose hi is not finite (values that are
+// infinite or NaN, or too large to sum in FP32) is summed again term by term
+// in FP64.  FP64 storage sums its pairs and groups in FP64.
+//   Measured, one lbm_conserved call (about 50 us of it the host's wait):
+// D2Q37 FP32 2048^2 2133 -> 281 us, FP16 storage 2075 -> 225 us, D3Q107 FP32
+// 128 x 128 x 127 3354 -> 396 us.  With 4-byte loads, each used as it
+// arrives, the first took 735 us: too few bytes in flight.
 // ---------------------------------------------------------------------------
 constexpr int kRedThreads = 256;
-constexpr int kRedMaxBlocks = 1024;
+constexpr int kRedMaxBlocks = 1024;  // partials an instance has room for
+constexpr int kRedBlocks = 6 * 152;    // blocks of a large grid: whole waves of 2, 3 or 6 blocks on each of 152 SMs
 constexpr int kRedVals = 5;  // mass, momentum[3], energy
+constexpr int kTotalsRun = 16;
 
 __device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll
@@ -1507,28 +1585,197 @@ __device__ __forceinline__ double warp_sum(double v) {
   return v;
 }
 
+// hi + lo += x, the error of the addition to hi kept in lo
+__device__ __forceinline__ void two_sum(float& hi, float& lo, float x) {
+  const float s = __fadd_rn(hi, x), b = __fsub_rn(s, hi);
+  lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, b)), __fsub_rn(x, b)));
+  hi = s;
+}
+__device__ __forceinline__ void two_sum(f32x2& hi, f32x2& lo, f32x2 x) {
+  const f32x2 s = add_f32x2(hi, x), b = sub_f32x2(s, hi);
+  lo = add_f32x2(lo, add_f32x2(sub_f32x2(hi, sub_f32x2(s, b)), sub_f32x2(x, b)));
+  hi = s;
+}
+
+// the totals of the cells begin, begin + stride, ... below end, every term
+// added in FP64
 template <int LAT, class S>
-__global__ void __launch_bounds__(kRedThreads) k_conserve_partial(const S* __restrict__ src, long long N,
-                                                                   const Args<double> a, const Args<float> af,
-                                                                   double* __restrict__ partial) {
+__device__ __noinline__ void add_totals_by_term(const S* __restrict__ src, long long ps, long long begin,
+                                                long long end, long long stride, double r, double half_r2,
+                                                const Args<float>& af, double (&acc)[kRedVals]) {
   using L = Lat<LAT>;
-  constexpr int Q = L::Q;
-  const long long ps = a.ps;
-  double acc[kRedVals] = {0.0, 0.0, 0.0, 0.0, 0.0};
-  for (long long cell = (long long)blockIdx.x * blockDim.x + threadIdx.x; cell < N;
-       cell += (long long)gridDim.x * blockDim.x) {
-    static_for<Q>([&](auto I) {
+  for (long long cell = begin; cell < end; cell += stride) {
+    static_for<L::Q>([&](auto I) {
       constexpr int i = decltype(I)::value;
-      double gi, hi;
-      decode_pair_d<Q, S>(src, i, ps, cell, L::grp(i), af, gi, hi);
-      acc[0] += gi;
-      if constexpr (L::cx(i) != 0) acc[1] += (a.r * L::cx(i)) * gi;
-      if constexpr (L::cy(i) != 0) acc[2] += (a.r * L::cy(i)) * gi;
-      if constexpr (L::cz(i) != 0) acc[3] += (a.r * L::cz(i)) * gi;
-      acc[4] += a.half_r2 * L::c2(i) * gi + hi;
+      float gf, hf;
+      ld_gh<L::Q, S, float>(src, i, ps, cell, gf, hf);
+      scale_gh<S, float>(gf, hf, L::grp(i), af);
+      const double g = gf;
+      acc[0] += g;
+      if constexpr (L::cx(i) != 0) acc[1] += (r * L::cx(i)) * g;
+      if constexpr (L::cy(i) != 0) acc[2] += (r * L::cy(i)) * g;
+      if constexpr (L::cz(i) != 0) acc[3] += (r * L::cz(i)) * g;
+      acc[4] += half_r2 * L::c2(i) * g + double(hf);
     });
   }
-  __shared__ double sh[kRedThreads / 32][kRedVals];
+}
+
+// adds the deviations' totals of the VEC cells from begin, from begin +
+// stride, ... below end: acc = {mass, momentum[3], energy}.  VEC = 4 (FP32
+// and 16-bit storage) reads 16 bytes at a time: src, ps, begin and stride
+// are multiples of four elements, and so is end.
+template <int LAT, class S, int VEC>
+__device__ __forceinline__ void add_totals(const S* __restrict__ src, long long ps, long long begin, long long end,
+                                           long long stride, double r, double half_r2, const Args<float>& af,
+                                           double (&acc)[kRedVals]) {
+  using L = Lat<LAT>;
+  constexpr int Q = L::Q, G = L::G, D = L::D;
+  if constexpr (sizeof(S) == 8) {
+    for (long long cell = begin; cell < end; cell += stride) {
+      double g0, h0;
+      ld_gh<Q, S, double>(src, 0, ps, cell, g0, h0);
+      double mass = g0, hs = h0, k2 = 0.0, grp = 0.0, j[3] = {0.0, 0.0, 0.0};
+      static_for<Q>([&](auto I) {
+        constexpr int i = decltype(I)::value;
+        if constexpr (i % 2 == 1) {  // the pair c, -c
+          double gp, hp, gm, hm;
+          ld_gh<Q, S, double>(src, i, ps, cell, gp, hp);
+          ld_gh<Q, S, double>(src, i + 1, ps, cell, gm, hm);
+          const double d = gp - gm;
+          if constexpr (L::cx(i) != 0) j[0] = fma(double(L::cx(i)), d, j[0]);
+          if constexpr (L::cy(i) != 0) j[1] = fma(double(L::cy(i)), d, j[1]);
+          if constexpr (L::cz(i) != 0) j[2] = fma(double(L::cz(i)), d, j[2]);
+          hs += hp + hm;
+          grp += gp + gm;
+          if constexpr (i + 2 >= Q || L::grp(i + 2 < Q ? i + 2 : i) != L::grp(i)) {  // the group's last pair
+            mass += grp;
+            k2 = fma(double(L::c2(i)), grp, k2);
+            grp = 0.0;
+          }
+        }
+      });
+      acc[0] += mass;
+#pragma unroll
+      for (int a = 0; a < D; ++a) acc[1 + a] = fma(r, j[a], acc[1 + a]);
+      acc[4] += fma(half_r2, k2, hs);
+    }
+  } else {
+    // V cells per load (16 bytes per thread and load keep enough of them in
+    // flight); the cells' values are summed in the two halves of f32x2
+    constexpr int V = VEC;
+    using W = typename std::conditional<V == 4, uint4, unsigned>::type;
+    auto value = [](unsigned w) { return __uint_as_float(w); };
+    while (begin < end) {
+      const long long first = begin;
+      f32x2 hi[G], lo[G], jhi[D][3], jlo[D][3], hhi = 0, hlo = 0;
+#pragma unroll
+      for (int g = 0; g < G; ++g) hi[g] = lo[g] = 0ull;
+#pragma unroll
+      for (int a = 0; a < D; ++a)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) jhi[a][c] = jlo[a][c] = 0ull;
+      auto add = [&](auto I, f32x2 g, f32x2 h) {
+        constexpr int i = decltype(I)::value;
+        if constexpr (IsS16<S>::value) {  // the 16-bit codec in FP32, as the step evaluates it
+          float a0, a1;
+          unpack_f32x2(g, a0, a1);
+          g = pack_f32x2(__fmul_rn(a0, af.gref[L::grp(i)]), __fmul_rn(a1, af.gref[L::grp(i)]));
+          unpack_f32x2(h, a0, a1);
+          h = pack_f32x2(__fmul_rn(a0, af.hscale[L::grp(i)]), __fmul_rn(a1, af.hscale[L::grp(i)]));
+        }
+        two_sum(hi[L::grp(i)], lo[L::grp(i)], g);
+        two_sum(hhi, hlo, h);
+        auto axis = [&](int a, int c) {
+          if (c > 0) two_sum(jhi[a][c - 1], jlo[a][c - 1], g);
+          if (c < 0) two_sum(jhi[a][-c - 1], jlo[a][-c - 1], neg_f32x2(g));
+        };
+        axis(0, L::cx(i));
+        axis(1, L::cy(i));
+        if constexpr (D == 3) axis(2, L::cz(i));
+      };
+#pragma unroll 1
+      for (int k = 0; k < kTotalsRun / V && begin < end; ++k, begin += stride) {
+        // the next directions' loads are issued before the present ones are summed
+        constexpr int B = V == 4 ? 3 : 8, NB = (Q + B - 1) / B, NPL = IsS16<S>::value ? 1 : 2;
+        W buf[2][B][NPL];
+        auto fetch = [&](auto K) {
+          static_for<B>([&](auto J) {
+            constexpr int i = decltype(K)::value * B + decltype(J)::value;
+            if constexpr (i < Q) {
+#pragma unroll
+              for (int q = 0; q < NPL; ++q)
+                buf[decltype(K)::value % 2][decltype(J)::value][q] =
+                    ld_again(reinterpret_cast<const W*>(reinterpret_cast<const unsigned*>(src) + ((size_t)(q * Q + i) * ps + begin)));
+            }
+          });
+        };
+        fetch(std::integral_constant<int, 0>{});
+        static_for<NB>([&](auto K) {
+          constexpr int kk = decltype(K)::value;
+          if constexpr (kk + 1 < NB) fetch(std::integral_constant<int, kk + 1>{});
+          static_for<B>([&](auto J) {
+            constexpr int i = kk * B + decltype(J)::value;
+            if constexpr (i < Q) {
+              const W(&w)[NPL] = buf[kk % 2][decltype(J)::value];
+              auto two = [&](unsigned g0, unsigned g1, unsigned h0, unsigned h1) {
+                if constexpr (IsS16<S>::value) {
+                  float ga, ha, gb, hb;
+                  unpack16<S>(g0, ga, ha);
+                  unpack16<S>(g1, gb, hb);
+                  add(std::integral_constant<int, i>{}, pack_f32x2(ga, gb), pack_f32x2(ha, hb));
+                } else {
+                  add(std::integral_constant<int, i>{}, pack_f32x2(value(g0), value(g1)), pack_f32x2(value(h0), value(h1)));
+                }
+              };
+              if constexpr (V == 4) {
+                two(w[0].x, w[0].y, w[NPL - 1].x, w[NPL - 1].y);
+                two(w[0].z, w[0].w, w[NPL - 1].z, w[NPL - 1].w);
+              } else {
+                two(w[0], 0u, w[NPL - 1], 0u);
+              }
+            }
+          });
+        });
+      }
+      bool fine = true;
+      auto total = [&](f32x2 h2, f32x2 l2) {
+        float h0, h1, l0, l1;
+        unpack_f32x2(h2, h0, h1);
+        unpack_f32x2(l2, l0, l1);
+        fine = fine && isfinite(h0) && isfinite(h1);
+        return (double(h0) + double(l0)) + (double(h1) + double(l1));
+      };
+      double part[kRedVals] = {0.0, 0.0, 0.0, 0.0, total(hhi, hlo)};
+      static_for<G>([&](auto K) {
+        constexpr int g = decltype(K)::value;
+        constexpr int c2 = (LAT == 0 ? kD2Q37 : kD3Q107).c2[g];
+        const double m = total(hi[g], lo[g]);
+        part[0] += m;
+        part[4] = fma(half_r2 * c2, m, part[4]);
+      });
+#pragma unroll
+      for (int a = 0; a < D; ++a) {
+        double j = 0.0;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) j = fma(double(c + 1), total(jhi[a][c], jlo[a][c]), j);
+        part[1 + a] = r * j;
+      }
+      if (!fine) {
+#pragma unroll
+        for (int k = 0; k < kRedVals; ++k) part[k] = 0.0;
+        for (int v = 0; v < V; ++v)
+          add_totals_by_term<LAT, S>(src, ps, first + v, begin, stride, r, half_r2, af, part);
+      }
+#pragma unroll
+      for (int k = 0; k < kRedVals; ++k) acc[k] += part[k];
+    }
+  }
+}
+
+// the block's sum of acc, in warp order, into partial[blockIdx.x]
+template <int THREADS>
+__device__ __forceinline__ void store_block_totals(const double (&acc)[kRedVals], double* __restrict__ partial) {
+  __shared__ double sh[THREADS / 32][kRedVals];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
   for (int k = 0; k < kRedVals; ++k) {
@@ -1538,9 +1785,27 @@ __global__ void __launch_bounds__(kRedThreads) k_conserve_partial(const S* __res
   __syncthreads();
   if (threadIdx.x < kRedVals) {
     double s = 0.0;
-    for (int w = 0; w < kRedThreads / 32; ++w) s += sh[w][threadIdx.x];
+    for (int w = 0; w < THREADS / 32; ++w) s += sh[w][threadIdx.x];
     partial[blockIdx.x * kRedVals + threadIdx.x] = s;
   }
+}
+
+template <int LAT, class S>
+__global__ void __launch_bounds__(kRedThreads, 2) k_conserve_partial(const S* __restrict__ src, long long N,
+                                                                   const Args<double> a, const Args<float> af,
+                                                                   double* __restrict__ partial) {
+  double acc[kRedVals] = {0.0, 0.0, 0.0, 0.0, 0.0};
+  // an instance's planes start on 256 bytes, so whole quads of cells can be
+  // read at once; the last N mod 4 go to the first threads of the last block
+  constexpr int V = sizeof(S) == 8 ? 1 : 4;
+  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x, nt = (long long)gridDim.x * blockDim.x;
+  const long long whole = N / V * V;
+  add_totals<LAT, S, V>(src, a.ps, t * V, whole, nt * V, a.r, a.half_r2, af, acc);
+  if constexpr (V > 1) {
+    if (blockIdx.x == gridDim.x - 1)
+      add_totals<LAT, S, 1>(src, a.ps, whole + threadIdx.x, N, kRedThreads, a.r, a.half_r2, af, acc);
+  }
+  store_block_totals<kRedThreads>(acc, partial);
 }
 
 

@@ -152,7 +152,7 @@ cudaError_t launch_conserve(const Instance* I, const void* src, double* partial,
 
 int reduction_blocks(long long N) {
   long long b = (N + kRedThreads - 1) / kRedThreads;
-  if (b > kRedMaxBlocks) b = kRedMaxBlocks;
+  if (b > kRedBlocks) b = kRedBlocks;
   if (b < 1) b = 1;
   return (int)b;
 }

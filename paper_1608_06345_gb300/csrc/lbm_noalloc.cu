@@ -57,40 +57,23 @@ int scratch_on_current_device(double** out) {
 }
 
 // Partial sums of the deviations over one contiguous chunk of cells per block.
-template <int LAT, class S>
-__global__ void __launch_bounds__(kNaThreads) k_conserve_chunk(const S* __restrict__ src, long long N, long long ps,
+// VEC = 4: 16-byte loads, for states and plane strides that are multiples of
+// four 4-byte words
+template <int LAT, class S, int VEC>
+__global__ void __launch_bounds__(kNaThreads, 2) k_conserve_chunk(const S* __restrict__ src, long long N, long long ps,
                                                                 double r, double half_r2, const Args<float> af,
                                                                 double* __restrict__ partial) {
-  using L = Lat<LAT>;
-  constexpr int Q = L::Q;
   double acc[kRedVals] = {0.0, 0.0, 0.0, 0.0, 0.0};
   const long long begin = (long long)blockIdx.x * kNaCellsPerBlock;
   const long long end = (begin + kNaCellsPerBlock < N) ? begin + kNaCellsPerBlock : N;
-  for (long long cell = begin + threadIdx.x; cell < end; cell += kNaThreads) {
-    static_for<Q>([&](auto I) {
-      constexpr int i = decltype(I)::value;
-      double gi, hi;
-      decode_pair_d<Q, S>(src, i, ps, cell, L::grp(i), af, gi, hi);
-      acc[0] += gi;
-      if constexpr (L::cx(i) != 0) acc[1] += (r * L::cx(i)) * gi;
-      if constexpr (L::cy(i) != 0) acc[2] += (r * L::cy(i)) * gi;
-      if constexpr (L::cz(i) != 0) acc[3] += (r * L::cz(i)) * gi;
-      acc[4] += half_r2 * L::c2(i) * gi + hi;
-    });
+  if constexpr (VEC == 4) {
+    const long long whole = begin + (end - begin) / 4 * 4;
+    add_totals<LAT, S, 4>(src, ps, begin + 4 * threadIdx.x, whole, 4 * kNaThreads, r, half_r2, af, acc);
+    add_totals<LAT, S, 1>(src, ps, whole + threadIdx.x, end, kNaThreads, r, half_r2, af, acc);
+  } else {
+    add_totals<LAT, S, 1>(src, ps, begin + threadIdx.x, end, kNaThreads, r, half_r2, af, acc);
   }
-  __shared__ double sh[kNaThreads / 32][kRedVals];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-  for (int k = 0; k < kRedVals; ++k) {
-    const double v = warp_sum(acc[k]);
-    if (lane == 0) sh[warp][k] = v;
-  }
-  __syncthreads();
-  if (threadIdx.x < kRedVals) {
-    double s = 0.0;
-    for (int w = 0; w < kNaThreads / 32; ++w) s += sh[w][threadIdx.x];
-    partial[blockIdx.x * kRedVals + threadIdx.x] = s;
-  }
+  store_block_totals<kNaThreads>(acc, partial);
 }
 
 // Totals of the nblocks partials written by this call (one warp per value,
@@ -108,8 +91,15 @@ __global__ void k_conserve_chunk_final(const double* __restrict__ partial, int n
 template <int LAT, class S>
 cudaError_t launch_chunk(const void* state, long long N, long long ps, double r, double half_r2,
                          const Args<float>& af, double* scratch, int nblocks, cudaStream_t st) {
-  k_conserve_chunk<LAT, S><<<nblocks, kNaThreads, 0, st>>>(static_cast<const S*>(state), N, ps, r, half_r2, af,
-                                                           scratch);
+  if constexpr (sizeof(S) < 8) {
+    if (reinterpret_cast<uintptr_t>(state) % 16 == 0 && ps % 4 == 0) {
+      k_conserve_chunk<LAT, S, 4><<<nblocks, kNaThreads, 0, st>>>(static_cast<const S*>(state), N, ps, r, half_r2,
+                                                                  af, scratch);
+      return cudaGetLastError();
+    }
+  }
+  k_conserve_chunk<LAT, S, 1><<<nblocks, kNaThreads, 0, st>>>(static_cast<const S*>(state), N, ps, r, half_r2, af,
+                                                              scratch);
   return cudaGetLastError();
 }
 

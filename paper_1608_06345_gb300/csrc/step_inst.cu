@@ -1,7 +1,9 @@
 // Kernel instantiations and launchers of one (lattice, precision) pair,
 // selected at compile time by LBM_LAT (0 = D2Q37, 1 = D3Q107) and LBM_PREC
 // (0 = FP64, 1 = FP32, 2 = FP32 compute / FP16 storage, 3 = FP32 / BF16).
-// The build compiles this file once per pair so the objects build in parallel.
+// The build compiles this file once per pair and part, so that the objects
+// build in parallel: LBM_PART 0 the launcher table and the small kernels,
+// 1 the step's launch shapes, 2 the finite-difference step.
 #include "fd_march.cuh"
 
 #ifndef LBM_LAT
@@ -9,6 +11,9 @@
 #endif
 #ifndef LBM_PREC
 #error "LBM_PREC must be defined"
+#endif
+#ifndef LBM_PART
+#error "LBM_PART must be defined"
 #endif
 
 namespace lbm {
@@ -27,6 +32,22 @@ using StoreT = __nv_bfloat16;
 using ComputeT = float;
 #endif
 
+// instantiated in their own part only
+#if LBM_PART == 0
+#define LBM_STEP extern template
+#define LBM_FD extern template
+#elif LBM_PART == 1
+#define LBM_STEP template
+#define LBM_FD extern template
+#else
+#define LBM_STEP extern template
+#define LBM_FD template
+#endif
+LBM_STEP cudaError_t launch_step_plain<LBM_LAT, StoreT, ComputeT>(const Instance*, const void*, void*);
+LBM_STEP cudaError_t configure_step_t<LBM_LAT, StoreT, ComputeT>(const Instance*);
+LBM_FD cudaError_t launch_step_fd_any<LBM_LAT, StoreT, ComputeT>(const Instance*, const void*, void*, double);
+
+#if LBM_PART == 0
 #define LBM_CAT2(a, b, c) a##_##b##_##c
 #define LBM_CAT(a, b, c) LBM_CAT2(a, b, c)
 
@@ -44,5 +65,6 @@ extern const Launchers LBM_CAT(kLaunchers, LBM_LAT, LBM_PREC) = {
     &configure_step_t<LBM_LAT, StoreT, ComputeT>,
     &launch_step_fd_any<LBM_LAT, StoreT, ComputeT>,
 };
+#endif
 
 }  // namespace lbm
