@@ -44,9 +44,8 @@ enum lbm_status {
   LBM_ENOMEM = 2,     /* device or host allocation failed, or caller buffer too small */
   LBM_ECUDA = 3,      /* a CUDA runtime call failed */
   LBM_ENONFINITE = 4, /* a step produced a non-finite density or temperature */
-  LBM_ETIMEOUT = 5,   /* reserved for a bounded device-side wait that gives up; no
-                         kernel of this library waits on the device, so no call
-                         returns it */
+  LBM_ETIMEOUT = 5,   /* a bounded wait inside the two-step kernel (lbm_step) gave
+                         up after about a second: the state is not valid */
   LBM_EBUSY = 6       /* a pool's memory budget is full */
 };
 
@@ -124,7 +123,9 @@ int lbm_init_device(lbm_handle h, const double* rho, const double* u, const doub
  * which the time mapping of Sec. V implies).  Asynchronous on the instance's
  * stream.  Runs of at least twice the graph
  * length (lbm_set_graph_steps, default 64) replay a captured CUDA graph of
- * that many steps instead of launching each step; the arithmetic is the same. */
+ * that many steps instead of launching each step, and large D2Q37 grids with
+ * FP32 storage take two steps per launch; the arithmetic is the same, bit for
+ * bit. */
 int lbm_step(lbm_handle h, long n);
 
 /* Steps per CUDA graph replay of lbm_step (even, 0..4096); 0 launches every

@@ -572,23 +572,13 @@ __device__ __forceinline__ void moments_finish(const C (&acc)[5], const Args<C>&
 // cell whose equilibrium coefficients k (formed from its moments by
 // eq_coeffs) are known; cell is the element index within a plane (32 bits:
 // below 2^32 cells per instance)
-template <int LAT, class S, class C, bool IDX32, bool FD, int IB = 0, int IE = Lat<LAT>::Q, class GetG, class GetH,
-          class Conv>
-__device__ __forceinline__ void relax_store_k(GetG&& getg, GetH&& geth, Conv&& conv, const Args<C>& a,
-                                              const EqCoef<LAT, C>& k, S* __restrict__ dst, long long ps,
-                                              unsigned cell) {
+// relax_put_k: the same with put(I, g, h) receiving the new values (16-bit
+// storage: before packing) instead of the store
+template <int LAT, class S, class C, bool FD, int IB, int IE, class GetG, class GetH, class Conv, class Put>
+__device__ __forceinline__ void relax_put_k(GetG&& getg, GetH&& geth, Conv&& conv, const Args<C>& a,
+                                            const EqCoef<LAT, C>& k, Put&& put) {
   using L = Lat<LAT>;
-  constexpr int Q = L::Q;
   constexpr bool SCALED = IsS16<S>::value;
-  // IDX32: element index plane * ps + cell in unsigned 32 bits (the caller
-  // checked that every element index is below 2^32); else plane base + the
-  // cell's byte offset in 64 bits
-  char* db = reinterpret_cast<char*>(dst) + (size_t)cell * sizeof(S);
-  const size_t pb = (size_t)ps * sizeof(S);
-  auto st = [&](int plane, S v) {
-    if constexpr (IDX32) dst[(unsigned)plane * (unsigned)ps + cell] = v;
-    else *reinterpret_cast<S*>(db + (size_t)plane * pb) = v;
-  };
   const C hA = a.omega_g * a.half_delta * k.T;
   const C om1 = C(1) - a.omega_g;
   const C hbs = a.omega_g * a.half_delta * k.dT;
@@ -610,11 +600,7 @@ __device__ __forceinline__ void relax_store_k(GetG&& getg, GetH&& geth, Conv&& c
         dn -= cv.g;
         en -= cv.h;
       }
-      // one 32-bit (g_i, h_i) pair
-      unsigned* dp = reinterpret_cast<unsigned*>(dst);
-      const unsigned pv = pack16<S>(static_cast<float>(dn), static_cast<float>(en));
-      if constexpr (IDX32) dp[(unsigned)i * (unsigned)ps + cell] = pv;
-      else dp[(size_t)i * ps + cell] = pv;
+      put(I, dn, en);
     } else {
       C gn = fma(a.omega_f, dF - gi, gi);
       C hn = fma(hA, dF, fma(om1, hi, hbs * a.gref[g]));
@@ -623,6 +609,34 @@ __device__ __forceinline__ void relax_store_k(GetG&& getg, GetH&& geth, Conv&& c
         gn -= cv.g;
         hn -= cv.h;
       }
+      put(I, gn, hn);
+    }
+  });
+}
+
+template <int LAT, class S, class C, bool IDX32, bool FD, int IB = 0, int IE = Lat<LAT>::Q, class GetG, class GetH,
+          class Conv>
+__device__ __forceinline__ void relax_store_k(GetG&& getg, GetH&& geth, Conv&& conv, const Args<C>& a,
+                                              const EqCoef<LAT, C>& k, S* __restrict__ dst, long long ps,
+                                              unsigned cell) {
+  constexpr int Q = Lat<LAT>::Q;
+  // IDX32: element index plane * ps + cell in unsigned 32 bits (the caller
+  // checked that every element index is below 2^32); else plane base + the
+  // cell's byte offset in 64 bits
+  char* db = reinterpret_cast<char*>(dst) + (size_t)cell * sizeof(S);
+  const size_t pb = (size_t)ps * sizeof(S);
+  auto st = [&](int plane, S v) {
+    if constexpr (IDX32) dst[(unsigned)plane * (unsigned)ps + cell] = v;
+    else *reinterpret_cast<S*>(db + (size_t)plane * pb) = v;
+  };
+  relax_put_k<LAT, S, C, FD, IB, IE>(getg, geth, conv, a, k, [&](auto I, C gn, C hn) {
+    constexpr int i = decltype(I)::value;
+    if constexpr (IsS16<S>::value) {  // one 32-bit (g_i, h_i) pair
+      unsigned* dp = reinterpret_cast<unsigned*>(dst);
+      const unsigned pv = pack16<S>(static_cast<float>(gn), static_cast<float>(hn));
+      if constexpr (IDX32) dp[(unsigned)i * (unsigned)ps + cell] = pv;
+      else dp[(size_t)i * ps + cell] = pv;
+    } else {
       st(i, static_cast<S>(gn));
       st(Q + i, static_cast<S>(hn));
     }
@@ -1373,6 +1387,216 @@ __global__ void __launch_bounds__(BX, MINB) k_step_mirror(const S* __restrict__ 
     relax(e + o, getg(k), geth(k), gn, hn);
     if (active) store(i, (unsigned)half, gn, hn);
   });
+}
+
+// ---------------------------------------------------------------------------
+// two steps of a D2Q37 FP32 grid in one launch
+//
+// A single step of a large grid runs at the memory's copy rate (1433 us per
+// 4096^2 step, 1.02 of it), so what is left is to move the state less often.
+// A block marches down a strip of columns.  Two of its four groups of warps
+// (A) do the first step, one row after the other, and put the new
+// populations into shared memory; the other two (B) do the second step a few
+// rows behind, from there, and store the result.  The state between the two
+// steps never leaves the SM: a cell costs one read and one write of its
+// populations per two steps.
+//   Ring: the population of direction i of row r is pulled by row r + c_y,
+// so it is kept until B has pulled that row: c_y + 5 rows, 5 on average over
+// the lattice, 189 KB at 128 columns, one block per SM.  The directions of
+// one c_y share a region [row slot][plane][column].
+//   Order: A's groups take the even and the odd rows, B's likewise, so that
+// one group's loads overlap the other's arithmetic (16 warps of 128
+// registers).  A stores row t once B has pulled row t - 8 of the band, B
+// pulls row q once A's rows up to q + 6 are stored; both wait on mbarriers.
+//   A's columns are the strip's w and 3 on each side, its rows the band's
+// and 3 above and below, each mapped to a grid cell by the axis' rule
+// (wrapped, or the edge cell's again at a zero-gradient end), so B pulls
+// without any boundary case.  Neighbouring strips repeat those cells' first
+// step.  Every cell's arithmetic is that of the single step, bit for bit.
+//   Measured, us per step, single -> pair: 4096^2 1433 -> 1144, 2048^2 361 ->
+// 284, 1024^2 92.6 -> 77.5, 2999 x 1777 519 -> 377.  It is bound by A's wait
+// for its loads (5000 of a group's 10000 cycles per row).  Also built: one
+// group each for A and B with the next row's loads in registers (255 of
+// them) and a block barrier per row, 1521 us; A's loads by cp.async into
+// shared memory two rows ahead, 96 columns, 12 warps, 1156; two columns per
+// thread in f32x2 arithmetic, 0.64 of the instructions but 8 warps, 1387;
+// rows brought to L2 ahead of the loads, 1400 - 1500.
+// ---------------------------------------------------------------------------
+constexpr int kPairW = 128;           // A's columns
+constexpr int kPairOut = kPairW - 6;  // columns a strip can hold
+
+struct PairRing {
+  static constexpr int cy(int i) { return Lat<0>::cy(i); }
+  static constexpr int depth(int k) { return k + 2; }  // rows kept of the directions with c_y = k - 3
+  static constexpr int members(int k) {
+    int n = 0;
+    for (int i = 0; i < 37; ++i) n += cy(i) == k - 3;
+    return n;
+  }
+  static constexpr int rank(int i) {
+    int n = 0;
+    for (int j = 0; j < i; ++j) n += cy(j) == cy(i);
+    return n;
+  }
+  // words per column of one row slot, and the region's first word per column
+  static constexpr int row(int k, int planes) { return members(k) * planes; }
+  static constexpr int begin(int k, int planes) {
+    int n = 0;
+    for (int j = 0; j < k; ++j) n += row(j, planes) * depth(j);
+    return n;
+  }
+  static constexpr size_t bytes(int planes) { return sizeof(unsigned) * kPairW * (size_t)begin(7, planes); }
+};
+
+__device__ __forceinline__ int map_coord(int q, int n, int bc) {
+  if (bc == kPeriodic) {
+    while (q < 0) q += n;
+    while (q >= n) q -= n;
+    return q;
+  }
+  return q < 0 ? 0 : (q > n - 1 ? n - 1 : q);
+}
+
+// mbarriers of the ring (one arrival per warp of a group); a wait gives up
+// after about a second, so that no fault elsewhere can leave a block spinning
+constexpr int kWaitTries = 1 << 20;
+
+__device__ __forceinline__ void bar_init(unsigned long long* b, unsigned count) {
+  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"((unsigned)__cvta_generic_to_shared(b)), "r"(count));
+}
+__device__ __forceinline__ void bar_arrive(unsigned long long* b) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"((unsigned)__cvta_generic_to_shared(b)) : "memory");
+}
+__device__ __forceinline__ bool bar_wait(unsigned long long* b, unsigned parity) {
+  const unsigned at = (unsigned)__cvta_generic_to_shared(b);
+  unsigned done = 0;
+  for (int n = 0; n < kWaitTries && !done; ++n)
+    asm volatile(
+        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, 1000;\n selp.u32 %0, 1, 0, p;\n}"
+        : "=r"(done)
+        : "r"(at), "r"(parity)
+        : "memory");
+  return __all_sync(0xffffffffu, done != 0);
+}
+
+template <bool IDX32>
+__global__ void __launch_bounds__(4 * kPairW, 1) k_step_pair(const float* __restrict__ src, float* __restrict__ dst,
+                                                             const Args<float> a, int w) {
+  using L = Lat<0>;
+  using S = float;
+  using C = float;
+  constexpr int Q = L::Q, W = kPairW, NPL = 2, NB = 8;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ unsigned long long stored[NB], pulled[NB];  // A's row t, B's row q (mod NB)
+  S* ring = reinterpret_cast<S*>(smem_raw);
+  const int nx = a.n[0], ny = a.n[1];
+  const int x0 = blockIdx.x * w;
+  const int y0 = (int)((long long)ny * blockIdx.y / gridDim.y), y1 = (int)((long long)ny * (blockIdx.y + 1) / gridDim.y);
+  const int rows = y1 - y0;
+  const long long ps = a.ps;
+  const int j = threadIdx.x & (W - 1), group = threadIdx.x / W;  // 0, 1: A's even and odd rows; 2, 3: B's
+  if (threadIdx.x < NB) {
+    bar_init(stored + threadIdx.x, W / 32);
+    bar_init(pulled + threadIdx.x, W / 32);
+  }
+  __syncthreads();
+  auto arrive = [&](unsigned long long* b) {
+    __syncwarp();
+    if ((threadIdx.x & 31) == 0) bar_arrive(b);
+  };
+  auto wait = [&](unsigned long long* b, int n) {  // for row n's arrivals
+    const bool ok = bar_wait(b + (n & (NB - 1)), (n / NB) & 1);
+    if (!ok) atomicOr(a.flag, 2u);
+    return ok;
+  };
+  // first word (of column 0) of the slot of A's row t in the region of c_y = k - 3, and that two rows later
+  auto slot_of = [](auto K, int t) {
+    constexpr int k = decltype(K)::value;
+    constexpr int step = PairRing::row(k, NPL) * W, first = PairRing::begin(k, NPL) * W, d = PairRing::depth(k);
+    return first + (t % d) * step;
+  };
+  auto two_later = [](auto K, int s) {
+    constexpr int k = decltype(K)::value;
+    constexpr int step = PairRing::row(k, NPL) * W, end = PairRing::begin(k + 1, NPL) * W;
+    s += 2 * step;
+    return s >= end ? s - step * PairRing::depth(k) : s;
+  };
+  int slot[7];
+  if (group < 2) {
+    const bool active = j < w + 6;
+    const int mine = rows + 6;  // the band's rows and 3 on each side
+    unsigned xb[7];
+    {
+      const int x = map_coord(x0 - 3 + j, nx, a.bc[0]);
+#pragma unroll
+      for (int k = 0; k < 7; ++k) xb[k] = (unsigned)pull_coord(x, k - 3, nx, a.bc[0]);
+    }
+    static_for<7>([&](auto K) { slot[decltype(K)::value] = slot_of(K, group); });
+    for (int t = group; t < mine; t += 2) {
+      C g[Q], h[Q];
+      if (active) {
+        const int y = map_coord(y0 - 3 + t, ny, a.bc[1]);
+        unsigned yo[7];
+#pragma unroll
+        for (int k = 0; k < 7; ++k) yo[k] = (unsigned)pull_coord(y, k - 3, ny, a.bc[1]) * (unsigned)nx;
+        static_for<Q>([&](auto I) {
+          constexpr int i = decltype(I)::value;
+          auto at = [&](int plane) {
+            if constexpr (IDX32) return src + (size_t)((unsigned)plane * (unsigned)ps + yo[L::cy(i) + 3] + xb[L::cx(i) + 3]);
+            else return src + ((size_t)plane * (size_t)ps + yo[L::cy(i) + 3] + xb[L::cx(i) + 3]);
+          };
+          g[i] = __ldg(at(i));
+          h[i] = __ldg(at(Q + i));
+        });
+      }
+      auto getg = [&](auto I) { return g[decltype(I)::value]; };
+      auto geth = [&](auto I) { return h[decltype(I)::value]; };
+      EqCoef<0, C> k;
+      if (active) {
+        C drho, u[3], dT;
+        moments_raw<0, C, false>(getg, geth, a, drho, u, dT);
+        if (!(isfinite(drho) && isfinite(dT))) atomicOr(a.flag, 1u);
+        eq_coeffs<0, C>(drho, u, dT, a, k);
+      }
+      // the rows this one replaces were last pulled by B's row t - 8; the band's
+      // first rows replace none, but must not overtake the other group's
+      if (t >= 8 ? !wait(pulled, t - 8) : t >= 3 && !wait(stored, t - 3)) return;
+      if (active)
+        relax_put_k<0, S, C, false, 0, Q>(getg, geth, [](auto) { return ConvGH<C>{C(0), C(0)}; }, a, k,
+                                          [&](auto I, C gn, C hn) {
+                                            constexpr int i = decltype(I)::value, kc = L::cy(i) + 3;
+                                            constexpr int pl = NPL * PairRing::rank(i);
+                                            S* p = ring + slot[kc] + j;
+                                            p[pl * W] = gn;
+                                            p[(pl + 1) * W] = hn;
+                                          });
+      arrive(stored + (t & (NB - 1)));
+      static_for<7>([&](auto K) { slot[decltype(K)::value] = two_later(K, slot[decltype(K)::value]); });
+    }
+  } else {
+    const bool active = j < w && x0 + j < nx;
+    // B's row q pulls direction i from A's row q + 3 - c_y
+    static_for<7>([&](auto K) { slot[decltype(K)::value] = slot_of(K, group - 2 + 6 - decltype(K)::value); });
+    int seen = 0;  // A's rows known to be stored
+    for (int q = group - 2; q < rows; q += 2) {
+      for (; seen <= q + 6; ++seen)
+        if (!wait(stored, seen)) return;
+      C g[Q], h[Q];
+      static_for<Q>([&](auto I) {
+        constexpr int i = decltype(I)::value, kc = L::cy(i) + 3;
+        constexpr int pl = NPL * PairRing::rank(i);
+        const S* p = ring + slot[kc] + (active ? j : 0) + 3 - L::cx(i);
+        g[i] = p[pl * W];
+        h[i] = p[(pl + 1) * W];
+      });
+      arrive(pulled + (q & (NB - 1)));
+      if (active)
+        collide_store<0, S, C, IDX32>([&](auto I) { return g[decltype(I)::value]; },
+                                      [&](auto I) { return h[decltype(I)::value]; }, a, dst, ps,
+                                      (unsigned)nx * (unsigned)(y0 + q) + (unsigned)(x0 + j));
+      static_for<7>([&](auto K) { slot[decltype(K)::value] = two_later(K, slot[decltype(K)::value]); });
+    }
+  }
 }
 
 // ---------------------------------------------------------------------------

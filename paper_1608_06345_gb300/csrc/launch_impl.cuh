@@ -259,10 +259,101 @@ cudaError_t launch_step_shape(const Instance* inst, const void* src, void* dst, 
   }
 }
 
-// sets the shape's kernel attributes on the current device without
-// launching (done before a graph capture)
+// ---------------------------------------------------------------------------
+// two steps in one launch
+// ---------------------------------------------------------------------------
+inline int device_sms() {
+  static std::atomic<int> sms[64];
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev >= 64) return 152;
+  int n = sms[dev].load(std::memory_order_relaxed);
+  if (n == 0) {
+    if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 152;
+    sms[dev].store(n, std::memory_order_relaxed);
+  }
+  return n;
+}
+
+// Strips of columns and bands of rows: one block fits an SM, a block's time
+// is that of its rows + 7 iterations, so take the number of bands with the
+// fewest iterations over all waves.  Returns the share of them that a grid of
+// full strips without those 7 would need.
+inline double pair_grid(const Instance* inst, int* strips, int* bands, int* width) {
+  const int nx = inst->n[0], ny = inst->n[1], sms = device_sms();
+  *strips = (nx + kPairOut - 1) / kPairOut;
+  *width = (nx + *strips - 1) / *strips;
+  long long best = -1;
+  *bands = 1;
+  for (int nb = 1; nb <= ny && nb <= 512; ++nb) {
+    const long long waves = ((long long)*strips * nb + sms - 1) / sms;
+    const long long cost = waves * ((ny + nb - 1) / nb + 7);
+    if (best < 0 || cost < best) {
+      best = cost;
+      *bands = nb;
+    }
+  }
+  return (double)inst->N / ((double)kPairOut * sms * (double)best);
+}
+
+// Whether two steps per launch are the faster way.  Measured against the
+// share of pair_grid: 0.44 (384^2) 0.79 of the single step's speed, 0.57
+// (512^2) 1.03, 0.60 (100 x 6000) 1.18, 0.72 (768^2) 1.15, 0.80 (1024^2)
+// 1.19, 0.94 (4096^2) 1.25.
+template <int LAT, class S, class C>
+bool has_pair_t(const Instance* inst) {
+  if constexpr (LAT == 0 && std::is_same<S, float>::value) {
+    int strips, bands, width;
+    return pair_grid(inst, &strips, &bands, &width) >= 0.6;
+  } else {
+    return false;
+  }
+}
+
+template <bool IDX32>
+cudaError_t launch_pair_v(const Instance* inst, const void* src, void* dst, bool configure_only) {
+  auto kern = k_step_pair<IDX32>;
+  constexpr size_t smem = PairRing::bytes(2);
+  static std::atomic<unsigned long long> configured{0};
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (dev >= 64 || !(configured.load(std::memory_order_acquire) & (1ull << dev))) {
+    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    if (dev < 64) configured.fetch_or(1ull << dev, std::memory_order_release);
+  }
+  if (configure_only) return cudaSuccess;
+  int strips, bands, width;
+  pair_grid(inst, &strips, &bands, &width);
+  kern<<<dim3((unsigned)strips, (unsigned)bands), 4 * kPairW, smem, inst->stream>>>(
+      static_cast<const float*>(src), static_cast<float*>(dst), inst->af, width);
+  return cudaGetLastError();
+}
+
+template <int LAT, class S, class C>
+cudaError_t launch_pair_t(const Instance* inst, const void* src, void* dst, bool configure_only) {
+  if constexpr (LAT == 0 && std::is_same<S, float>::value) {
+    if (2LL * Lat<LAT>::Q * inst->ps < (1LL << 32)) return launch_pair_v<true>(inst, src, dst, configure_only);
+    return launch_pair_v<false>(inst, src, dst, configure_only);
+  } else {
+    return cudaErrorInvalidConfiguration;
+  }
+}
+
+template <int LAT, class S, class C>
+cudaError_t launch_step_pair(const Instance* inst, const void* src, void* dst) {
+  return launch_pair_t<LAT, S, C>(inst, src, dst, false);
+}
+
+// sets the kernel attributes of the shape, and of the two-step kernel where
+// the instance takes it, on the current device without launching (done
+// before a graph capture)
 template <int LAT, class S, class C>
 cudaError_t configure_step_t(const Instance* inst) {
+  if (has_pair_t<LAT, S, C>(inst)) {
+    const cudaError_t e = launch_pair_t<LAT, S, C>(inst, nullptr, nullptr, true);
+    if (e != cudaSuccess) return e;
+  }
   return launch_step_shape<LAT, S, C>(inst, nullptr, nullptr, true);
 }
 

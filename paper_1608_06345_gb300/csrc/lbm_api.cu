@@ -157,12 +157,25 @@ int reduction_blocks(long long N) {
   return (int)b;
 }
 
+// Enqueues the next step, or the next two in one launch where the instance
+// takes that way (pairs) and n >= 2, from buffer *cur; returns the steps
+// taken, or 0 with *e set.
+int advance_once(const Instance* I, int* cur, long n, bool pairs, cudaError_t* e) {
+  const bool pair = pairs && n >= 2;
+  *e = pair ? launchers_of(I).step_pair(I, I->buf[*cur], I->buf[1 - *cur])
+            : launch_step(I, I->buf[*cur], I->buf[1 - *cur]);
+  if (*e != cudaSuccess) return 0;
+  *cur ^= 1;
+  return pair ? 2 : 1;
+}
+
 // Reads the error word (synchronising the stream) and maps it to a status.
 int check_status(Instance* I) {
   unsigned int flag = 0;
   cudaError_t e = cudaMemcpyAsync(&flag, I->flag, sizeof(flag), cudaMemcpyDeviceToHost, I->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(I->stream);
   if (e != cudaSuccess) return cuda_fail(e, "synchronising the instance stream");
+  if (flag & 2u) return fail(LBM_ETIMEOUT, "a wait inside the two-step kernel gave up; the state is not valid");
   if (flag & 1u) return fail(LBM_ENONFINITE, "a step met a non-finite density or temperature");
   return LBM_OK;
 }
@@ -254,11 +267,12 @@ cudaError_t capture_graph(Instance* I) {
   e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
   cudaError_t le = cudaSuccess;
   if (e == cudaSuccess) {
-    int c = I->cur;
-    for (int k = 0; k < I->graph_steps && le == cudaSuccess; ++k) {
-      le = launch_step(I, I->buf[c], I->buf[1 - c]);
-      c ^= 1;
-    }
+    // the launches swap the buffers an even number of times: the last two
+    // steps of graph_steps = 4 m + 2 are single ones
+    const bool pairs = launchers_of(I).has_pair(I);
+    int c = I->cur, left = I->graph_steps;
+    while (left > 0 && le == cudaSuccess)
+      left -= advance_once(I, &c, left, pairs && (left > 2 || I->graph_steps % 4 == 0), &le);
     cudaGraph_t g = nullptr;
     e = cudaStreamEndCapture(cs, &g);
     if (e == cudaSuccess && le == cudaSuccess) {
@@ -415,11 +429,13 @@ int lbm_step(lbm_handle h, long n) {
       h->steps_done += h->graph_steps;
     }
   }
-  for (long k = 0; k < n; ++k) {
-    cudaError_t e = launch_step(h, h->buf[h->cur], h->buf[1 - h->cur]);
+  const bool pairs = h->graph_steps > 0 && n >= 2 && launchers_of(h).has_pair(h);
+  while (n > 0) {
+    cudaError_t e;
+    const int k = advance_once(h, &h->cur, n, pairs, &e);
     if (e != cudaSuccess) return cuda_fail(e, "launching the step kernel");
-    h->cur ^= 1;
-    ++h->steps_done;
+    n -= k;
+    h->steps_done += k;
   }
   return LBM_OK;
 }

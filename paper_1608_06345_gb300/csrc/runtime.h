@@ -83,6 +83,8 @@ struct Launchers {
   void (*shape_get)(int k, int* stage, int* bx);
   cudaError_t (*configure)(const Instance* inst);
   cudaError_t (*step_fd)(const Instance* inst, const void* src, void* dst, double lam);
+  bool (*has_pair)(const Instance* inst);  // whether two steps in one launch are the faster way here
+  cudaError_t (*step_pair)(const Instance* inst, const void* src, void* dst);
 };
 
 extern const Launchers kLaunchers_0_0, kLaunchers_0_1, kLaunchers_0_2, kLaunchers_0_3;

@@ -44,6 +44,7 @@ using ComputeT = float;
 #define LBM_FD template
 #endif
 LBM_STEP cudaError_t launch_step_plain<LBM_LAT, StoreT, ComputeT>(const Instance*, const void*, void*);
+LBM_STEP cudaError_t launch_step_pair<LBM_LAT, StoreT, ComputeT>(const Instance*, const void*, void*);
 LBM_STEP cudaError_t configure_step_t<LBM_LAT, StoreT, ComputeT>(const Instance*);
 LBM_FD cudaError_t launch_step_fd_any<LBM_LAT, StoreT, ComputeT>(const Instance*, const void*, void*, double);
 
@@ -64,6 +65,8 @@ extern const Launchers LBM_CAT(kLaunchers, LBM_LAT, LBM_PREC) = {
     &shape_get_t<LBM_LAT, StoreT>,
     &configure_step_t<LBM_LAT, StoreT, ComputeT>,
     &launch_step_fd_any<LBM_LAT, StoreT, ComputeT>,
+    &has_pair_t<LBM_LAT, StoreT, ComputeT>,
+    &launch_step_pair<LBM_LAT, StoreT, ComputeT>,
 };
 #endif
 
