@@ -1672,6 +1672,104 @@ __global__ void __launch_bounds__(BX) k_step_fd(const S* __restrict__ src, S* __
 }
 
 // ---------------------------------------------------------------------------
+// the same in two passes over a tile of BX x BY x BZ cells per block: the
+// moments from the cell's own 2Q values, then for each direction the own
+// value again, its upwind neighbours, the relaxation and the store; value by
+// value the arithmetic of k_step_fd.  Nothing but the moments is held between
+// the passes, so many more cells are in flight, and a tile's neighbours along
+// y and z are mostly its own cells, found in L1.
+//   Measured, us per step, against k_step_fd: D3Q107 (255 registers and
+// spills, 8 warps per SM; the loads of 1460 neighbours per cell went to L2)
+// 112 x 96 x 80 FP32 2069 -> 800, FP16 storage 940 -> 731; 256 x 128 x 128
+// 9879 -> 3820 and 5543 -> 3488.  D2Q37 FP16 storage 4096^2 1789 -> 1537,
+// FP32 2613 -> 2690, which keeps k_step_fd; D3Q107 FP64 256 x 128 x 128 33.8
+// -> 31.2 ms.  Also tried: tiles of 32 x 4 x 4 and 32 x 2 x 4, 0 to 10% more;
+// the second pass as a loop over the pairs with the next direction's loads
+// ahead, 883 (112 x 96 x 80 FP32); that in f32x2 arithmetic, two cells per
+// thread, 693, but with other roundings.
+// ---------------------------------------------------------------------------
+template <int LAT, class S, class C, int BX, int BY, int BZ, int MINB>
+__global__ void __launch_bounds__(BX* BY* BZ, MINB) k_step_fd_tile(const S* __restrict__ src, S* __restrict__ dst,
+                                                                    const Args<C> a, C lamr) {
+  using L = Lat<LAT>;
+  constexpr int Q = L::Q;
+  const int x = blockIdx.x * BX + threadIdx.x, y = blockIdx.y * BY + threadIdx.y;
+  const int z = (L::D == 3) ? blockIdx.z * BZ + threadIdx.z : 0;
+  const int nx = a.n[0], ny = a.n[1], nz = a.n[2];
+  if (x >= nx || y >= ny || z >= nz) return;
+  const unsigned row = (unsigned)nx * ((unsigned)y + (unsigned)ny * (unsigned)z);
+  const unsigned cell = (unsigned)x + row;
+  // element index of the cell at p + k, k = -2, -1, 1, 2 along each axis, after the boundary rule
+  unsigned at[3][4];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    const int k = j < 2 ? j - 2 : j - 1;
+    at[0][j] = row + (unsigned)pull_coord(x, -k, nx, a.bc[0]);
+    at[1][j] = (unsigned)x + (unsigned)nx * ((unsigned)pull_coord(y, -k, ny, a.bc[1]) + (unsigned)ny * (unsigned)z);
+    at[2][j] = (L::D == 3) ? (unsigned)x + (unsigned)nx * ((unsigned)y + (unsigned)ny * (unsigned)pull_coord(z, -k, nz, a.bc[2])) : 0u;
+  }
+  const long long ps = a.ps;
+  auto plane = [&](int i) {
+    if constexpr (IsS16<S>::value) return reinterpret_cast<const unsigned*>(src) + (size_t)i * ps;
+    else return src + (size_t)i * ps;
+  };
+  auto split = [&](auto v, C& g, C& h) {
+    float lo, hi;
+    unpack16<S>(v, lo, hi);
+    g = static_cast<C>(lo);
+    h = static_cast<C>(hi);
+  };
+  auto near = [&](int i, unsigned e, C& g, C& h) {
+    if constexpr (IsS16<S>::value) {
+      split(__ldg(plane(i) + e), g, h);
+    } else {
+      g = __ldg(plane(i) + e);
+      h = __ldg(plane(Q + i) + e);
+    }
+  };
+  C drho, u[3], dT;
+  {
+    C g, h;
+    moments_raw<LAT, C, IsS16<S>::value>(
+        [&](auto I) { near(decltype(I)::value, cell, g, h); return g; },
+        [&](auto I) { near(decltype(I)::value, cell, g, h); return h; }, a, drho, u, dT);
+  }
+  if (!(isfinite(drho) && isfinite(dT))) atomicOr(a.flag, 1u);
+  C g, h;  // the direction's own values
+  auto own = [&](auto I) {
+    constexpr int i = decltype(I)::value;
+    if constexpr (IsS16<S>::value) {
+      split(ld_again(plane(i) + cell), g, h);
+    } else {
+      g = ld_again(plane(i) + cell);
+      h = ld_again(plane(Q + i) + cell);
+    }
+    return g;
+  };
+  auto conv = [&](auto I) {
+    constexpr int i = decltype(I)::value;
+    C cg = C(0), ch = C(0);
+    auto axis = [&](int ax, int c) {
+      if (c == 0) return;
+      C gm2, hm2, gm1, hm1, gp1, hp1;  // the upwind-2, upwind-1 and downwind-1 values
+      near(i, at[ax][c > 0 ? 0 : 3], gm2, hm2);
+      near(i, at[ax][c > 0 ? 1 : 2], gm1, hm1);
+      near(i, at[ax][c > 0 ? 2 : 1], gp1, hp1);
+      const C sg = c > 0 ? C(1) : C(-1);
+      const C dg = sg * (gm2 - C(6) * gm1 + C(3) * g + C(2) * gp1) * C(1.0 / 6.0);
+      const C dh = sg * (hm2 - C(6) * hm1 + C(3) * h + C(2) * hp1) * C(1.0 / 6.0);
+      cg = fma(C(c), dg, cg);
+      ch = fma(C(c), dh, ch);
+    };
+    axis(0, L::cx(i));
+    axis(1, L::cy(i));
+    axis(2, L::cz(i));
+    return ConvGH<C>{lamr * cg, lamr * ch};
+  };
+  relax_store<LAT, S, C, false, true>(own, [&](auto) { return h; }, conv, a, drho, u, dT, dst, ps, cell);
+}
+
+// ---------------------------------------------------------------------------
 // batched step of a pool of independent instances (continuous batching)
 //
 // Every resident instance has a slot descriptor in device memory (its

@@ -362,15 +362,48 @@ cudaError_t launch_step_plain(const Instance* inst, const void* src, void* dst) 
   return launch_step_shape<LAT, S, C>(inst, src, dst, false);
 }
 
-// the finite-difference step (lam = dt/dx): 128 cells per block in 2D, 64 in 3D
+// the finite-difference step (lam = dt/dx)
+template <int LAT, class S, class C, int BX, int BY, int BZ, int MINB>
+cudaError_t launch_step_fd_tile(const Instance* inst, const void* src, void* dst, double lam) {
+  const dim3 grid((unsigned)((inst->n[0] + BX - 1) / BX), (unsigned)((inst->n[1] + BY - 1) / BY),
+                  (unsigned)((inst->n[2] + BZ - 1) / BZ));
+  k_step_fd_tile<LAT, S, C, BX, BY, BZ, MINB><<<grid, dim3(BX, BY, BZ), 0, inst->stream>>>(
+      static_cast<const S*>(src), static_cast<S*>(dst), args_of<C>(inst), static_cast<C>(lam * inst->table.r));
+  return cudaGetLastError();
+}
+// one thread per cell holding its 2Q values, BX cells of a row per block
+template <int LAT, class S, class C, int BX>
+cudaError_t launch_step_fd_row(const Instance* inst, const void* src, void* dst, double lam) {
+  const dim3 grid((unsigned)((inst->n[0] + BX - 1) / BX), (unsigned)inst->n[1], (unsigned)inst->n[2]);
+  k_step_fd<LAT, S, C, BX><<<grid, BX, 0, inst->stream>>>(static_cast<const S*>(src), static_cast<S*>(dst),
+                                                          args_of<C>(inst), static_cast<C>(lam * inst->table.r));
+  return cudaGetLastError();
+}
+
+// The faster of the two per lattice, storage and size (large grids: figures at
+// k_step_fd_tile).  A tile's block is long and large, so grids of few tiles
+// leave SMs idle that the row kernel's smaller blocks would use; us per step,
+// tile and row: D3Q107 FP32 32^3 (64 tiles) 74 / 72, 40^3 (150) 97 / 127, 1000
+// x 4 x 4 (63) 59 / 37; FP16 storage 32^3 57 / 63; FP64 32^3 (128) 553 / 380,
+// 48^3 (432) 878 / 1238; D2Q37 FP16 storage 256^2 (256) 13.1 / 11.1, 512^2
+// (1024) 27.1 / 29.6.
 template <int LAT, class S, class C>
 cudaError_t launch_step_fd_t(const Instance* inst, const void* src, void* dst, double lam) {
-  constexpr int BX = (LAT == 0) ? 128 : 64;
-  const dim3 grid((unsigned)((inst->n[0] + BX - 1) / BX), (unsigned)inst->n[1], (unsigned)inst->n[2]);
-  const Args<C>& a = args_of<C>(inst);
-  k_step_fd<LAT, S, C, BX><<<grid, BX, 0, inst->stream>>>(static_cast<const S*>(src), static_cast<S*>(dst), a,
-                                                          static_cast<C>(lam * inst->table.r));
-  return cudaGetLastError();
+  auto tiles = [&](int bx, int by, int bz) {
+    return ((long long)inst->n[0] + bx - 1) / bx * ((inst->n[1] + by - 1) / by) * ((inst->n[2] + bz - 1) / bz);
+  };
+  if constexpr (LAT == 0) {
+    if constexpr (IsS16<S>::value)
+      if (tiles(32, 8, 1) >= 3 * 152) return launch_step_fd_tile<LAT, S, C, 32, 8, 1, 3>(inst, src, dst, lam);
+    return launch_step_fd_row<LAT, S, C, 128>(inst, src, dst, lam);
+  } else {
+    if constexpr (sizeof(S) == 8) {
+      if (tiles(16, 4, 4) >= 2 * 152) return launch_step_fd_tile<LAT, S, C, 16, 4, 4, 2>(inst, src, dst, lam);
+    } else {
+      if (tiles(16, 8, 4) >= 64) return launch_step_fd_tile<LAT, S, C, 16, 8, 4, 2>(inst, src, dst, lam);
+    }
+    return launch_step_fd_row<LAT, S, C, 64>(inst, src, dst, lam);
+  }
 }
 
 // pool: the shape of the batched step per (lattice, storage)
