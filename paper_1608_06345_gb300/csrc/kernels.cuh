@@ -63,6 +63,15 @@ struct Lat {
 };
 
 // ---------------------------------------------------------------------------
+// start of a kernel that may be set up while its stream's previous kernel
+// drains (launch_next): wait until that one has finished and its writes are
+// visible, before touching global memory
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ void wait_for_previous_kernel() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
+// ---------------------------------------------------------------------------
 // per-instance constants, already converted to the compute type C on the host
 // (a double->float conversion runs on the FP64 pipe, which is slow on GB300)
 // ---------------------------------------------------------------------------
@@ -983,6 +992,7 @@ __device__ __forceinline__ void boundary_row(int k, int ny, int nz, int& y, int&
 
 template <int LAT, class S, class C, int STAGE, int BX, int MINB = 1, bool IDX32 = false, int ROWS = kRowsAll>
 __global__ void __launch_bounds__(BX, MINB) k_step(const S* __restrict__ src, S* __restrict__ dst, const Args<C> a) {
+  wait_for_previous_kernel();
   const int x = blockIdx.x * BX + threadIdx.x;
   if constexpr (ROWS == kRowsInterior) {
     step_cell<LAT, S, C, STAGE, BX, IDX32, true>(src, dst, a, x, blockIdx.y + 3, blockIdx.z + 3);
@@ -1041,6 +1051,7 @@ __global__ void __launch_bounds__(32 * P, MINB) k_step_split(const S* __restrict
   constexpr int K = SP::kmax();
   constexpr bool SCALED = IsS16<S>::value;
   __shared__ C red[P][5][32];
+  wait_for_previous_kernel();
   const int lane = threadIdx.x, w = threadIdx.y;
   const int nx = a.n[0], ny = a.n[1], nz = a.n[2];
   const int x = blockIdx.x * 32 + lane, y = blockIdx.y, z = blockIdx.z;
@@ -1153,6 +1164,7 @@ __global__ void __launch_bounds__(BX, MINB) k_step_mirror(const S* __restrict__ 
   constexpr bool SCALED = IsS16<S>::value;
   static_assert(BX % 32 == 0, "whole warps");
   static_assert(!(HS && SCALED), "16-bit pairs are held packed in registers");
+  wait_for_previous_kernel();
   const int lane = threadIdx.x & 31;
   const int half = lane >> 4;
   const int nx = a.n[0], ny = a.n[1], nz = a.n[2];
@@ -1488,6 +1500,7 @@ __global__ void __launch_bounds__(4 * kPairW, 1) k_step_pair(const float* __rest
   constexpr int Q = L::Q, W = kPairW, NPL = 2, NB = 8;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ unsigned long long stored[NB], pulled[NB];  // A's row t, B's row q (mod NB)
+  wait_for_previous_kernel();
   S* ring = reinterpret_cast<S*>(smem_raw);
   const int nx = a.n[0], ny = a.n[1];
   const int x0 = blockIdx.x * w;
@@ -1614,6 +1627,7 @@ __global__ void __launch_bounds__(BX) k_step_fd(const S* __restrict__ src, S* __
                                                 C lamr) {
   using L = Lat<LAT>;
   constexpr int Q = L::Q;
+  wait_for_previous_kernel();
   const int x = blockIdx.x * BX + threadIdx.x;
   const int y = blockIdx.y, z = blockIdx.z;
   const int nx = a.n[0], ny = a.n[1], nz = a.n[2];
@@ -1694,6 +1708,7 @@ __global__ void __launch_bounds__(BX* BY* BZ, MINB) k_step_fd_tile(const S* __re
   using L = Lat<LAT>;
   constexpr int Q = L::Q;
   const int x = blockIdx.x * BX + threadIdx.x, y = blockIdx.y * BY + threadIdx.y;
+  wait_for_previous_kernel();
   const int z = (L::D == 3) ? blockIdx.z * BZ + threadIdx.z : 0;
   const int nx = a.n[0], ny = a.n[1], nz = a.n[2];
   if (x >= nx || y >= ny || z >= nz) return;
@@ -1793,6 +1808,7 @@ struct PoolSlot {
 template <int LAT, class S, class C, int STAGE, int BX>
 __global__ void __launch_bounds__(BX) k_pool_step(const PoolSlot<C>* __restrict__ slots,
                                                   const int4* __restrict__ tiles, const int* __restrict__ n_tiles) {
+  wait_for_previous_kernel();
   const int nt = *n_tiles;
   for (int t = blockIdx.x; t < nt; t += gridDim.x) {
     const int4 tl = tiles[t];  // slot, x0, y, z
@@ -1806,6 +1822,7 @@ __global__ void __launch_bounds__(BX) k_pool_step(const PoolSlot<C>* __restrict_
 
 template <class C>
 __global__ void k_pool_advance(PoolSlot<C>* __restrict__ slots, int nslots) {
+  wait_for_previous_kernel();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < nslots && slots[i].steps_left > 0) {
     if (*slots[i].a.flag) {
