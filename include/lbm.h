@@ -231,8 +231,8 @@ int lbm_conserved_noalloc(int lattice, int prec, double gamma, double rho0, doub
                           long long ncells, long long plane_stride, void* stream, double* out);
 
 /* Launch shapes of the step kernel (execution control with no counterpart in
- * the paper; every shape computes the same step, the stage-4, 7 and 8
- * shapes up to the summation order of the moments).  Each (lattice, precision) has a small
+ * the paper; every shape computes the same step, the FP32 and 16-bit
+ * stage-4, 7 and 8 shapes up to the summation order of the moments).  Each (lattice, precision) has a small
  * table of compiled candidates (how the pulled values are staged --
  * registers, shared memory by cp.async, g in registers and h in shared
  * memory (stages 0-3), the velocities of each cell split over 4 warps
@@ -241,7 +241,8 @@ int lbm_conserved_noalloc(int lattice, int prec, double gamma, double rho0, doub
  * (stage 6) or half of them so and half in shared memory (stage 9), or two
  * lanes per cell, one for c and one for -c of every
  * (c, -c) pair, whose moment sums meet by warp shuffles (stage 8) -- and
- * the cells per thread block); index 0 is the default.
+ * the cells per thread block); index 0 is the default, which picks by the
+ * grid's size among kernels that give the same bits.
  * lbm_shape_info describes candidate `index` (LBM_EINVAL past the end). */
 int lbm_shape_info(int lattice, int prec, int index, int* stage, int* block);
 

@@ -94,7 +94,11 @@ struct Args {
   C pref[10];        // A0(u = 0, t0) - 1 per group
   // 16-bit storage codec: dg = gref * d, dh = hscale * e
   C inv_gref[10], hscale[10], inv_hscale[10];
-  unsigned int* flag;  // error word: bit 0 = non-finite rho or T met
+  unsigned int* flag;  // error word: bit 0 = non-finite rho or T met, bit 1 = a wait gave up
+  // FP64 relaxation (relax_put_k)
+  C om1_f;           // 1 - 1 / tau_f
+  C hd_fg;           // (delta / 2) tau_f / tau_g
+  C wf[10];          // group weights / tau_f
 };
 
 // ---------------------------------------------------------------------------
@@ -336,15 +340,16 @@ __device__ __forceinline__ void eq_coeffs(C drho, const C (&u)[3], C dT, const A
 // s.  Velocities are ordered by group, so a group's coefficients c0..c4 are
 // formed once, at its first pair in the range, and are dead after its last.
 // IB is 0 or odd, IE odd or Q (whole pairs only).
-template <int LAT, class C, int IB = 0, int IE = Lat<LAT>::Q, class Emit>
+// RELAX: emits omega_f dF_i
+template <int LAT, class C, int IB = 0, int IE = Lat<LAT>::Q, bool RELAX = false, class Emit>
 __device__ __forceinline__ void eq_emit(const EqCoef<LAT, C>& k, const Args<C>& a, Emit&& emit) {
   using L = Lat<LAT>;
   C c0, c1, c2, c3, c4;
   auto group = [&](int g) {
     const C x2 = a.x2g[g];
     const C P = fma(x2, fma(x2, k.pc, k.pb), k.pa);
-    const C W = a.wg[g] * k.rho;
-    c0 = a.wg[g] * fma(k.drho, C(1) + P, a.rho0 * (P - a.pref[g]));
+    const C W = (RELAX ? a.wf[g] : a.wg[g]) * k.rho;
+    c0 = (RELAX ? a.wf[g] : a.wg[g]) * fma(k.drho, C(1) + P, a.rho0 * (P - a.pref[g]));
     c1 = W * fma(k.be1, x2, k.be0);
     c2 = W * fma(k.ga1, x2, k.ga0);
     c3 = W * C(1.0 / 6.0);
@@ -486,6 +491,20 @@ __device__ __forceinline__ void moments_dev(GetG&& getg, GetH&& geth, const Args
   moments_raw<LAT, C, false>(getg, geth, a, drho, u, dT);
 }
 
+// the velocities in P parts of whole (c, -c) pairs
+template <int LAT, int P>
+struct Split {
+  static constexpr int NP = (Lat<LAT>::Q - 1) / 2;  // (c, -c) pairs
+  // part 0: the rest velocity and pairs [0, NP/P); part w: pairs [w NP/P, (w+1) NP/P)
+  __host__ __device__ static constexpr int begin(int w) { return w == 0 ? 0 : 1 + 2 * (w * NP / P); }
+  __host__ __device__ static constexpr int end(int w) { return 1 + 2 * ((w + 1) * NP / P); }
+  __host__ __device__ static constexpr int kmax() {
+    int m = 0;
+    for (int w = 0; w < P; ++w) m = (end(w) - begin(w) > m) ? end(w) - begin(w) : m;
+    return m;
+  }
+};
+
 // The sums of moments_raw restricted to the velocities [IB, IE) (whole
 // pairs): acc = {sum dg, sum c_x dg, sum c_y dg, sum c_z dg,
 // r^2/2 sum c^2 dg + sum dh}.  Summing the parts of a partition gives the
@@ -503,7 +522,7 @@ __device__ __forceinline__ void moments_partial(GetG&& getg, GetH&& geth, const 
       H = geth(std::integral_constant<int, 0>{});
     }
   }
-  C jx = C(0), jy = C(0), jz = C(0), k2 = C(0);
+  C jx = C(0), jy = C(0), jz = C(0), k2 = C(0), gs = C(0);
   C s1 = C(1), s2 = C(2), s3 = C(3), sc2 = C(0), sh = C(1);
   static_for<L::Q>([&](auto I) {
     constexpr int i = decltype(I)::value;
@@ -532,17 +551,28 @@ __device__ __forceinline__ void moments_partial(GetG&& getg, GetH&& geth, const 
         k2 = fma(sc2, sp, k2);
         H = fma(sh, hp, H);
       } else {
-        m += sp;
         if constexpr (L::cx(i) != 0) jx = fma(C(L::cx(i)), df, jx);
         if constexpr (L::cy(i) != 0) jy = fma(C(L::cy(i)), df, jy);
         if constexpr (L::cz(i) != 0) jz = fma(C(L::cz(i)), df, jz);
-        k2 = fma(C(L::c2(i)), sp, k2);
         H += hp;
+        if constexpr (std::is_same<C, double>::value) {  // the group first: one instruction less per pair
+          constexpr bool first = i == IB || i - 2 < IB || L::grp(i - 2) != g;
+          constexpr bool last = i + 2 >= IE || L::grp(i + 2 < L::Q ? i + 2 : i) != g;
+          gs = first ? sp : gs + sp;
+          if constexpr (last) {
+            m += gs;
+            k2 = fma(C(L::c2(i)), gs, k2);
+          }
+        } else {
+          m += sp;
+          k2 = fma(C(L::c2(i)), sp, k2);
+        }
       }
     }
   });
   (void)s2;
   (void)s3;
+  (void)gs;
   acc[0] = m;
   acc[1] = jx;
   acc[2] = jy;
@@ -588,9 +618,30 @@ __device__ __forceinline__ void relax_put_k(GetG&& getg, GetH&& geth, Conv&& con
                                             const EqCoef<LAT, C>& k, Put&& put) {
   using L = Lat<LAT>;
   constexpr bool SCALED = IsS16<S>::value;
-  const C hA = a.omega_g * a.half_delta * k.T;
   const C om1 = C(1) - a.omega_g;
   const C hbs = a.omega_g * a.half_delta * k.dT;
+  if constexpr (std::is_same<S, double>::value) {
+    // FP64 is bound by its pipe, 2 instructions per SM and clock: with
+    // omega_f in the group's weights g* = (1 - omega_f) g + omega_f dF is one
+    // instruction instead of two (with the moments' sums by group: D2Q37
+    // 1024^2 1101 -> 1035 us per step, D3Q107 256 x 128 x 128 12.7 -> 11.5 ms)
+    const C hA = a.hd_fg * k.T;
+    C hbg = C(0);
+    eq_emit<LAT, C, IB, IE, true>(k, a, [&](auto I, C dFw) {
+      constexpr int i = decltype(I)::value;
+      if constexpr (i == IB || L::grp(i == 0 ? 0 : i - 1) != L::grp(i)) hbg = hbs * a.gref[L::grp(i)];
+      C gn = fma(a.om1_f, getg(I), dFw);
+      C hn = fma(hA, dFw, fma(om1, geth(I), hbg));
+      if constexpr (FD) {
+        const auto cv = conv(I);
+        gn -= cv.g;
+        hn -= cv.h;
+      }
+      put(I, gn, hn);
+    });
+    return;
+  }
+  const C hA = a.omega_g * a.half_delta * k.T;
   C ig = C(1), hAs = hA, hbg = C(0);  // per-group: 1/gref, hA/hs, hbs gref/hs (16-bit)
   eq_emit<LAT, C, IB, IE>(k, a, [&](auto I, C dF) {
     constexpr int i = decltype(I)::value;
@@ -667,7 +718,20 @@ template <int LAT, class S, class C, bool IDX32, bool FD, class GetG, class GetH
 __device__ __forceinline__ void collide_store_impl(GetG&& getg, GetH&& geth, Conv&& conv, const Args<C>& a,
                                                    S* __restrict__ dst, long long ps, unsigned cell) {
   C drho, u[3], dT;
-  moments_raw<LAT, C, IsS16<S>::value>(getg, geth, a, drho, u, dT);
+  if constexpr (std::is_same<S, double>::value) {
+    // summed in the four parts of k_step_split, so that the FP64 shapes give the same bits
+    C sum[5];
+    static_for<4>([&](auto W) {
+      constexpr int w = decltype(W)::value;
+      C acc[5];
+      moments_partial<LAT, C, false, Split<LAT, 4>::begin(w), Split<LAT, 4>::end(w)>(getg, geth, a, acc);
+#pragma unroll
+      for (int k = 0; k < 5; ++k) sum[k] = w == 0 ? acc[k] : sum[k] + acc[k];
+    });
+    moments_finish<LAT, C>(sum, a, drho, u, dT);
+  } else {
+    moments_raw<LAT, C, IsS16<S>::value>(getg, geth, a, drho, u, dT);
+  }
   if (!(isfinite(drho) && isfinite(dT))) atomicOr(a.flag, 1u);
   relax_store<LAT, S, C, IDX32, FD>(getg, geth, conv, a, drho, u, dT, dst, ps, cell);
 }
@@ -1026,19 +1090,6 @@ __global__ void __launch_bounds__(BX, MINB) k_step(const S* __restrict__ src, S*
 // Each thread holds 2 (end - begin) values instead of 2Q, which keeps the
 // register count near that of the D2Q37 kernel for D3Q107.
 // ---------------------------------------------------------------------------
-template <int LAT, int P>
-struct Split {
-  static constexpr int NP = (Lat<LAT>::Q - 1) / 2;  // (c, -c) pairs
-  // part 0: the rest velocity and pairs [0, NP/P); part w: pairs [w NP/P, (w+1) NP/P)
-  __host__ __device__ static constexpr int begin(int w) { return w == 0 ? 0 : 1 + 2 * (w * NP / P); }
-  __host__ __device__ static constexpr int end(int w) { return 1 + 2 * ((w + 1) * NP / P); }
-  __host__ __device__ static constexpr int kmax() {
-    int m = 0;
-    for (int w = 0; w < P; ++w) m = (end(w) - begin(w) > m) ? end(w) - begin(w) : m;
-    return m;
-  }
-};
-
 // SHARE: warp 0 alone finishes the moments and forms the equilibrium
 // coefficients, which the other warps read from shared memory after a second
 // barrier (less arithmetic per cell; worth it where the FP64 pipe is the bound)

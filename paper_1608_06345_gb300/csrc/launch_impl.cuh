@@ -37,6 +37,18 @@ cudaError_t launch_next(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, 
   return cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
 }
 
+inline int device_sms() {
+  static std::atomic<int> sms[64];
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev >= 64) return 152;
+  int n = sms[dev].load(std::memory_order_relaxed);
+  if (n == 0) {
+    if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 152;
+    sms[dev].store(n, std::memory_order_relaxed);
+  }
+  return n;
+}
+
 // dynamic shared memory of a step shape: none (STAGE 0, 6), h only (STAGE 3),
 // g and h (STAGE 1, 2)
 template <int LAT, class S, int STAGE, int BX>
@@ -179,17 +191,19 @@ cudaError_t launch_step_mirror(const Instance* inst, const void* src, void* dst,
 //   D2Q37 FP32:        (0,128,4) (0,256,2) (0,64,8) (0,128,1)
 //   D2Q37 16-bit:      (6,128,8) (6,128,7) (6,128,6) (6,256,3) (0,128,4) (0,64,8)
 //   D2Q37 FP64:        (0,128,1) (0,256,1) (0,64,1)  (4,32,4)  (7,32,4)
-//   D3Q107 FP32:       (3,64,6)  (3,64,1)  (1,64,1)  (4,32,6)  (8,32,8)  (8,64,4)  (3,128,3)
+//   D3Q107 FP32:       (3,64,6)  (3,64,6)  (3,32,12) (4,32,6)  (8,32,8)  (8,64,4)  (3,128,3)
 //   D3Q107 FP64:       (1,64,1)  (4,32,3)  (4,32,2)  (7,32,3)
-//   D3Q107 16-bit:     (6,64,6)  (9,256,2) (2,64,1)  (4,32,6)  (8,32,10) (8,32,12) (6,128,3)
+//   D3Q107 16-bit:     (6,64,6)  (9,256,2) (6,32,12) (4,32,6)  (8,32,10) (8,32,12) (6,128,3)
 // Stage 4 is the velocity-split step: 4 warps per block of 32 cells; stage 7
 // the same with the per-cell coefficients formed once by warp 0 and shared.
 // Stage 8 is the mirror-pair step: two lanes per cell (c and -c of every
 // pair), h staged in shared memory for FP32.  Stage 9 holds half the 16-bit
-// pairs packed in registers and stages the other half in shared memory.  The moments of stages 4, 7
-// and 8 are summed in another order, so their results differ from the
-// other shapes' by rounding; the defaults (index 0) are the shapes the
-// batched pool uses, whose results are bitwise those of a lone instance.
+// pairs packed in registers and stages the other half in shared memory.  In FP32 the
+// moments of stages 4, 7 and 8 are summed in another order, so their results
+// differ from the other shapes' by rounding; in FP64 every shape sums them in
+// the order of stage 4.  Index 0 picks by the grid's size among shapes of one
+// rounding (launch_step_shape), the one the batched pool has, so a pooled
+// instance's result is bitwise that of a lone one.
 template <int LAT, class S>
 struct StepShapes {
   static constexpr int count =
@@ -198,9 +212,9 @@ struct StepShapes {
     static const int s2[4][3] = {{0, 128, 4}, {0, 256, 2}, {0, 64, 8}, {0, 128, 1}};
     static const int s2h[6][3] = {{6, 128, 8}, {6, 128, 7}, {6, 128, 6}, {6, 256, 3}, {0, 128, 4}, {0, 64, 8}};
     static const int s2d[5][3] = {{0, 128, 1}, {0, 256, 1}, {0, 64, 1}, {4, 32, 4}, {7, 32, 4}};
-    static const int s3f[7][3] = {{3, 64, 6}, {3, 64, 1}, {1, 64, 1}, {4, 32, 6}, {8, 32, 8}, {8, 64, 4}, {3, 128, 3}};
+    static const int s3f[7][3] = {{3, 64, 6}, {3, 64, 6}, {3, 32, 12}, {4, 32, 6}, {8, 32, 8}, {8, 64, 4}, {3, 128, 3}};
     static const int s3d[4][3] = {{1, 64, 1}, {4, 32, 3}, {4, 32, 2}, {7, 32, 3}};
-    static const int s3h[7][3] = {{6, 64, 6}, {9, 256, 2}, {2, 64, 1}, {4, 32, 6}, {8, 32, 10}, {8, 32, 12}, {6, 128, 3}};
+    static const int s3h[7][3] = {{6, 64, 6}, {9, 256, 2}, {6, 32, 12}, {4, 32, 6}, {8, 32, 10}, {8, 32, 12}, {6, 128, 3}};
     const int(*t)[3] = (LAT == 0) ? (sizeof(S) == 8 ? s2d : (sizeof(S) == 2 ? s2h : s2))
                                   : (sizeof(S) == 4 ? s3f : (sizeof(S) == 8 ? s3d : s3h));
     *stage = t[k][0];
@@ -218,6 +232,23 @@ void shape_get_t(int k, int* stage, int* bx) {
   StepShapes<LAT, S>::get(k, stage, bx, &minb);
 }
 
+// The default D3Q107 shape of FP32 and 16-bit storage.  Blocks of 32 cells
+// where they leave a seventh fewer threads past the row ends than blocks of
+// 64 (us per step, 64 and 32 cells: FP32 32^3 14.6 / 7.7, 96^3 291 / 271; at
+// 193 cells, 224 threads for 256, 860 / 856); else 128 cells with FP32 storage
+// where they pad no more (256 x 128 x 128 1221 -> 1190, 193 x 130 x 97 860 ->
+// 830, 112 x 96 x 80 286 -> 267).
+template <int LAT, class S, class C, int STAGE>
+cudaError_t launch_default_3d(const Instance* inst, const void* src, void* dst, const Args<C>& a,
+                              bool configure_only) {
+  auto padded = [&](int bx) { return (inst->n[0] + bx - 1) / bx * bx; };
+  if (7 * padded(32) <= 6 * padded(64))
+    return launch_step_t<LAT, S, C, STAGE, 32, 12>(inst, src, dst, a, configure_only);
+  if constexpr (sizeof(S) == 4)
+    if (padded(128) == padded(64)) return launch_step_t<LAT, S, C, STAGE, 128, 3>(inst, src, dst, a, configure_only);
+  return launch_step_t<LAT, S, C, STAGE, 64, 6>(inst, src, dst, a, configure_only);
+}
+
 template <int LAT, class S, class C>
 cudaError_t launch_step_shape(const Instance* inst, const void* src, void* dst, bool configure_only = false) {
   const Args<C>& a = args_of<C>(inst);
@@ -228,6 +259,14 @@ cudaError_t launch_step_shape(const Instance* inst, const void* src, void* dst, 
       case 2: return launch_step_t<LAT, S, C, 0, 64>(inst, src, dst, a, configure_only);
       case 3: return launch_step_split<LAT, S, C, 4, 4>(inst, src, dst, a, configure_only);
       case 4: return launch_step_split<LAT, S, C, 4, 4, true>(inst, src, dst, a, configure_only);
+      case 0:
+        // a tube of a few blocks waits on one thread's chain of 560 FP64
+        // instructions per cell: split it while every SM has at most two
+        // 32-cell blocks (1000 x 4: 22.6 -> 9.4 us; 1000 x 16, 512 blocks:
+        // 22.8 us, split 30.2)
+        if ((long long)((inst->n[0] + 31) / 32) * inst->n[1] <= 2LL * device_sms())
+          return launch_step_split<LAT, S, C, 4, 4>(inst, src, dst, a, configure_only);
+        return launch_step_t<LAT, S, C, 0, 128>(inst, src, dst, a, configure_only);
       default: return launch_step_t<LAT, S, C, 0, 128>(inst, src, dst, a, configure_only);
     }
   } else if constexpr (LAT == 0 && sizeof(S) == 2) {
@@ -248,30 +287,32 @@ cudaError_t launch_step_shape(const Instance* inst, const void* src, void* dst, 
     }
   } else if constexpr (sizeof(S) == 4) {
     switch (k) {
-      case 1: return launch_step_t<LAT, S, C, 3, 64>(inst, src, dst, a, configure_only);
-      case 2: return launch_step_t<LAT, S, C, 1, 64>(inst, src, dst, a, configure_only);
+      case 1: return launch_step_t<LAT, S, C, 3, 64, 6>(inst, src, dst, a, configure_only);
+      case 2: return launch_step_t<LAT, S, C, 3, 32, 12>(inst, src, dst, a, configure_only);
       case 3: return launch_step_split<LAT, S, C, 4, 6>(inst, src, dst, a, configure_only);
       case 4: return launch_step_mirror<LAT, S, C, 64, 8, true>(inst, src, dst, a, configure_only);
       case 5: return launch_step_mirror<LAT, S, C, 128, 4, true>(inst, src, dst, a, configure_only);
       case 6: return launch_step_t<LAT, S, C, 3, 128, 3>(inst, src, dst, a, configure_only);
-      default: return launch_step_t<LAT, S, C, 3, 64, 6>(inst, src, dst, a, configure_only);
+      default: return launch_default_3d<LAT, S, C, 3>(inst, src, dst, a, configure_only);
     }
   } else if constexpr (sizeof(S) == 8) {
     switch (k) {
       case 1: return launch_step_split<LAT, S, C, 4, 3>(inst, src, dst, a, configure_only);
       case 2: return launch_step_split<LAT, S, C, 4, 2>(inst, src, dst, a, configure_only);
       case 3: return launch_step_split<LAT, S, C, 4, 3, true>(inst, src, dst, a, configure_only);
-      default: return launch_step_t<LAT, S, C, 1, 64>(inst, src, dst, a, configure_only);
+      // the split with shared coefficients is the faster at every size: 1000 x
+      // 16 x 16 983 -> 779 us, 256 x 128 x 128 14.1 -> 12.7 ms, 32^3 273 -> 116
+      default: return launch_step_split<LAT, S, C, 4, 3, true>(inst, src, dst, a, configure_only);
     }
   } else {
     switch (k) {
       case 1: return launch_step_t<LAT, S, C, 9, 256, 2>(inst, src, dst, a, configure_only);
-      case 2: return launch_step_t<LAT, S, C, 2, 64>(inst, src, dst, a, configure_only);
+      case 2: return launch_step_t<LAT, S, C, 6, 32, 12>(inst, src, dst, a, configure_only);
       case 3: return launch_step_split<LAT, S, C, 4, 6>(inst, src, dst, a, configure_only);
       case 4: return launch_step_mirror<LAT, S, C, 64, 10, false>(inst, src, dst, a, configure_only);
       case 5: return launch_step_mirror<LAT, S, C, 64, 12, false>(inst, src, dst, a, configure_only);
       case 6: return launch_step_t<LAT, S, C, 6, 128, 3>(inst, src, dst, a, configure_only);
-      default: return launch_step_t<LAT, S, C, 6, 64, 6>(inst, src, dst, a, configure_only);
+      default: return launch_default_3d<LAT, S, C, 6>(inst, src, dst, a, configure_only);
     }
   }
 }
@@ -279,18 +320,6 @@ cudaError_t launch_step_shape(const Instance* inst, const void* src, void* dst, 
 // ---------------------------------------------------------------------------
 // two steps in one launch
 // ---------------------------------------------------------------------------
-inline int device_sms() {
-  static std::atomic<int> sms[64];
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev >= 64) return 152;
-  int n = sms[dev].load(std::memory_order_relaxed);
-  if (n == 0) {
-    if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 152;
-    sms[dev].store(n, std::memory_order_relaxed);
-  }
-  return n;
-}
-
 // Strips of columns and bands of rows: one block fits an SM, a block's time
 // is that of its rows + 7 iterations, so take the number of bands with the
 // fewest iterations over all waves.  Returns the share of them that a grid of
@@ -423,7 +452,7 @@ cudaError_t launch_step_fd_t(const Instance* inst, const void* src, void* dst, d
 // pool: the shape of the batched step per (lattice, storage)
 template <int LAT, class S>
 struct PoolShape {
-  static constexpr int kStage = (LAT == 0) ? 0 : (sizeof(S) == 4 ? 3 : (sizeof(S) == 8 ? 1 : 2));
+  static constexpr int kStage = (LAT == 0) ? 0 : (sizeof(S) == 4 ? 3 : (sizeof(S) == 8 ? 1 : 6));
   static constexpr int kBX = (LAT == 0) ? 128 : 64;
 };
 
