@@ -235,7 +235,7 @@ int lbm_conserved_noalloc(int lattice, int prec, double gamma, double rho0, doub
  * stage-4, 7 and 8 shapes up to the summation order of the moments).  Each (lattice, precision) has a small
  * table of compiled candidates (how the pulled values are staged --
  * registers, shared memory by cp.async, g in registers and h in shared
- * memory (stages 0-3), the velocities of each cell split over 4 warps
+ * memory (stages 0, 1 and 3), the velocities of each cell split over 4 warps
  * (stage 4; stage 7 with the per-cell equilibrium coefficients formed once
  * and shared), for 16-bit storage the (g, h) pairs held packed in registers
  * (stage 6) or half of them so and half in shared memory (stage 9), or two

@@ -762,7 +762,6 @@ __device__ __forceinline__ C raw_value(S v) {
 //   STAGE 0: the 2Q pulled values live in registers (D2Q37)
 //   STAGE 1: they are staged in shared memory by 4/8-byte cp.async (D3Q107,
 //            FP32/FP64 storage): no registers held while the loads fly
-//   STAGE 2: staged in shared memory by plain loads (D3Q107, 16-bit storage)
 //   STAGE 3: g in registers, h staged in shared memory by cp.async (D3Q107,
 //            FP32/FP64): half the shared memory per cell of STAGE 1
 //   STAGE 6: 16-bit storage, the Q pulled (g_i, h_i) pairs held packed in
@@ -978,49 +977,25 @@ __device__ __forceinline__ void step_cell(const S* __restrict__ src, S* __restri
                                      [&](auto I) { return static_cast<C>(shv[decltype(I)::value * BX + t]); }, a,
                                      dst, ps, cell);
   } else {
+    static_assert(STAGE == 1 && (sizeof(S) == 4 || sizeof(S) == 8), "cp.async needs 4- or 8-byte elements");
     extern __shared__ __align__(16) unsigned char smem_raw[];
     S* sg = reinterpret_cast<S*>(smem_raw);  // [2Q][BX]
     const int t = threadIdx.x;
     static_for<Q>([&](auto I) {
       constexpr int i = decltype(I)::value;
-      if constexpr (STAGE == 1) {
-        static_assert(sizeof(S) == 4 || sizeof(S) == 8, "cp.async needs 4- or 8-byte elements");
-        const unsigned sa0 = (unsigned)__cvta_generic_to_shared(sg + i * BX + t);
-        const unsigned sa1 = (unsigned)__cvta_generic_to_shared(sg + (Q + i) * BX + t);
-        asm volatile("cp.async.ca.shared.global [%0], [%1], %2;\n" ::"r"(sa0), "l"(pptr(i, I)), "n"(sizeof(S)));
-        asm volatile("cp.async.ca.shared.global [%0], [%1], %2;\n" ::"r"(sa1), "l"(pptr(Q + i, I)),
-                     "n"(sizeof(S)));
-      } else if constexpr (IsS16<S>::value) {  // the 32-bit (g_i, h_i) pair into slot [i][t]
-        reinterpret_cast<unsigned*>(smem_raw)[i * BX + t] = __ldg(reinterpret_cast<const unsigned*>(pptr(i, I)));
-      } else {
-        sg[i * BX + t] = ldg_s(reinterpret_cast<const S*>(pptr(i, I)));
-        sg[(Q + i) * BX + t] = ldg_s(reinterpret_cast<const S*>(pptr(Q + i, I)));
-      }
+      const unsigned sa0 = (unsigned)__cvta_generic_to_shared(sg + i * BX + t);
+      const unsigned sa1 = (unsigned)__cvta_generic_to_shared(sg + (Q + i) * BX + t);
+      asm volatile("cp.async.ca.shared.global [%0], [%1], %2;\n" ::"r"(sa0), "l"(pptr(i, I)), "n"(sizeof(S)));
+      asm volatile("cp.async.ca.shared.global [%0], [%1], %2;\n" ::"r"(sa1), "l"(pptr(Q + i, I)), "n"(sizeof(S)));
     });
-    if constexpr (STAGE == 1) asm volatile("cp.async.wait_all;\n" ::: "memory");
+    asm volatile("cp.async.wait_all;\n" ::: "memory");
     // each thread reads back only the slots it filled itself; the reads are
     // volatile so that each pass re-reads shared memory instead of holding
     // every staged value in registers
-    if constexpr (IsS16<S>::value) {
-      const volatile unsigned* sp = reinterpret_cast<const volatile unsigned*>(smem_raw);
-      collide_store<LAT, S, C, SIDX32>(
-          [&](auto I) {
-            float lo, hi;
-            unpack16<S>(sp[decltype(I)::value * BX + t], lo, hi);
-            return static_cast<C>(lo);
-          },
-          [&](auto I) {
-            float lo, hi;
-            unpack16<S>(sp[decltype(I)::value * BX + t], lo, hi);
-            return static_cast<C>(hi);
-          },
-          a, dst, ps, cell);
-    } else {
-      const volatile S* sgv = sg;
-      collide_store<LAT, S, C, SIDX32>(
-          [&](auto I) { return raw_value<S, C>(sgv[decltype(I)::value * BX + t]); },
-          [&](auto I) { return raw_value<S, C>(sgv[(Q + decltype(I)::value) * BX + t]); }, a, dst, ps, cell);
-    }
+    const volatile S* sgv = sg;
+    collide_store<LAT, S, C, SIDX32>(
+        [&](auto I) { return raw_value<S, C>(sgv[decltype(I)::value * BX + t]); },
+        [&](auto I) { return raw_value<S, C>(sgv[(Q + decltype(I)::value) * BX + t]); }, a, dst, ps, cell);
   }
 }
 
@@ -1039,7 +1014,12 @@ __device__ __forceinline__ void step_cell(const S* __restrict__ src, S* __restri
 //                  ROW path's code and block-uniform row shift tables (UNI)
 // A 3D grid launches kRowsUniform (FP32 storage) or kRowsInterior then
 // kRowsBoundary (16-bit storage), so each kernel carries one code path.
-constexpr int kRowsAll = 0, kRowsInterior = 1, kRowsBoundary = 2, kRowsUniform = 3;
+//   kRowsFlat:     the cells of a 2D grid in their order in memory (block
+//                  (x)), whatever row they are in: where rows are no multiple
+//                  of 32 cells, the stores of row-wise blocks straddle the
+//                  32-byte sectors and their last block is partly empty.  The
+//                  general addressing, one integer addition more per load.
+constexpr int kRowsAll = 0, kRowsInterior = 1, kRowsBoundary = 2, kRowsUniform = 3, kRowsFlat = 4;
 
 __device__ __forceinline__ void boundary_row(int k, int ny, int nz, int& y, int& z) {
   if (k < 6 * ny) {
@@ -1058,7 +1038,10 @@ template <int LAT, class S, class C, int STAGE, int BX, int MINB = 1, bool IDX32
 __global__ void __launch_bounds__(BX, MINB) k_step(const S* __restrict__ src, S* __restrict__ dst, const Args<C> a) {
   wait_for_previous_kernel();
   const int x = blockIdx.x * BX + threadIdx.x;
-  if constexpr (ROWS == kRowsInterior) {
+  if constexpr (ROWS == kRowsFlat) {
+    const int y = x / a.n[0];
+    if (y < a.n[1]) step_cell<LAT, S, C, STAGE, BX, IDX32, false>(src, dst, a, x - y * a.n[0], y, 0);
+  } else if constexpr (ROWS == kRowsInterior) {
     step_cell<LAT, S, C, STAGE, BX, IDX32, true>(src, dst, a, x, blockIdx.y + 3, blockIdx.z + 3);
   } else if constexpr (ROWS == kRowsUniform) {
     step_cell<LAT, S, C, STAGE, BX, true, true, true>(src, dst, a, x, blockIdx.y, blockIdx.z);

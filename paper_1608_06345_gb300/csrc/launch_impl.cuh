@@ -50,7 +50,7 @@ inline int device_sms() {
 }
 
 // dynamic shared memory of a step shape: none (STAGE 0, 6), h only (STAGE 3),
-// g and h (STAGE 1, 2)
+// g and h (STAGE 1)
 template <int LAT, class S, int STAGE, int BX>
 constexpr size_t step_smem() {
   if constexpr (STAGE == 9) return sizeof(unsigned) * (Lat<LAT>::Q - (Lat<LAT>::Q + 1) / 2) * BX;
@@ -124,6 +124,19 @@ cudaError_t launch_step_v(const Instance* inst, const void* src, void* dst, cons
       return launch_next(k_step<LAT, S, C, STAGE, BX, MINB, IDX32, kRowsBoundary>, dim3(gx, (unsigned)boundary_rows(ny, nz), 1), BX, smem, inst->stream,
                          s, d, a);
     }
+  }
+  if constexpr (Lat<LAT>::D == 2 && IDX32 && sizeof(S) < 8) {
+    // Rows that are no multiple of 32 cells.  FP32 storage: always (us per
+    // step, row-wise and flat: 300 x 7 2.9 / 2.8, 333^2 10.4 / 7.7, 500^2 25.3 /
+    // 24.6).  16-bit storage is near its issue bound, so only where the rows
+    // start off the 32-byte sectors (8 pairs) and the state leaves the 126 MB
+    // of L2: 2999 x 1777 275 / 252; 3000 x 1776, on the sectors, 246 / 252;
+    // 2999 x 100, in L2, 14.3 / 15.1.
+    const bool flat = IsS16<S>::value ? inst->n[0] % 8 != 0 && 2 * inst->buf_bytes > 126000000
+                                      : inst->n[0] % 32 != 0;
+    if (flat && inst->N <= 0x7fffffffLL - BX)
+      return launch_next(k_step<LAT, S, C, STAGE, BX, MINB, IDX32, kRowsFlat>,
+                         dim3((unsigned)((inst->N + BX - 1) / BX), 1, 1), BX, smem, inst->stream, s, d, a);
   }
   return launch_next(k_step<LAT, S, C, STAGE, BX, MINB, IDX32, kRowsAll>, dim3(gx, (unsigned)ny, (unsigned)nz), BX, smem, inst->stream,
                      s, d, a);

@@ -63,3 +63,20 @@ def test_pool_gives_the_bits_of_a_lone_instance(lat, prec, shapes):
         for a, b in zip(got, run(lat, prec, shape, bc, fields, 0)):
             assert np.array_equal(a, b)
     pool.close()
+
+
+@pytest.mark.parametrize("prec,shape", [(1, (33, 5)), (1, (127, 3)), (1, (1, 40)), (2, (1003, 431)), (3, (433, 1001))])
+def test_cells_in_memory_order_give_the_bits_of_the_pool(prec, shape):
+    """Rows that are no multiple of 32 cells run as one flat range of cells
+    (16-bit storage: off the sectors and larger than L2); the pool works row
+    by row."""
+    from paper_1608_06345_gb300 import lbm
+    fields = li.random_fields(int(np.prod(shape)), 2, seed=sum(shape), u_amp=0.02)
+    pool = lbm.Pool(0, prec, budget_bytes=256 << 20, max_instances=2, bundle_steps=5)
+    ticket = pool.submit(1.4, 0.6, 0.7, shape, (1, 0), fields, 5)
+    pool.run(1)
+    pool.sync()
+    rc, got = pool.result(ticket, int(np.prod(shape)))
+    pool.close()
+    for a, b in zip(got, run(0, prec, shape, (1, 0), fields, 0, steps=5)):
+        assert np.array_equal(a, b)
