@@ -1839,8 +1839,8 @@ struct PoolSlot {
   int steps_left;  // steps still to take
 };
 
-template <int LAT, class S, class C, int STAGE, int BX>
-__global__ void __launch_bounds__(BX) k_pool_step(const PoolSlot<C>* __restrict__ slots,
+template <int LAT, class S, class C, int STAGE, int BX, int MINB>
+__global__ void __launch_bounds__(BX, MINB) k_pool_step(const PoolSlot<C>* __restrict__ slots,
                                                   const int4* __restrict__ tiles, const int* __restrict__ n_tiles) {
   wait_for_previous_kernel();
   const int nt = *n_tiles;

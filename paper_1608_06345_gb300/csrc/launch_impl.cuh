@@ -467,12 +467,16 @@ template <int LAT, class S>
 struct PoolShape {
   static constexpr int kStage = (LAT == 0) ? 0 : (sizeof(S) == 4 ? 3 : (sizeof(S) == 8 ? 1 : 6));
   static constexpr int kBX = (LAT == 0) ? 128 : 64;
+  // resident blocks per SM asked of the compiler, as in the step's shapes
+  // (D2Q37 FP32 took 138 registers, 3 blocks; 20 tubes of up to 12000 x 4 cells
+  // served in 11.0 -> 10.4 ms with 4)
+  static constexpr int kMinB = sizeof(S) == 8 ? 1 : (LAT == 0 ? 4 : 6);
 };
 
 template <int LAT, class S, class C>
 cudaError_t launch_pool_step_t(const PoolLaunch& pl) {
   using PS = PoolShape<LAT, S>;
-  auto kern = k_pool_step<LAT, S, C, PS::kStage, PS::kBX>;
+  auto kern = k_pool_step<LAT, S, C, PS::kStage, PS::kBX, PS::kMinB>;
   // the shared-memory opt-in was set by pool_grid_t at pool creation (outside
   // any stream capture)
   const size_t smem = step_smem<LAT, S, PS::kStage, PS::kBX>();
@@ -492,7 +496,7 @@ template <int LAT, class S, class C>
 int pool_grid_t() {
   using PS = PoolShape<LAT, S>;
   const size_t smem = step_smem<LAT, S, PS::kStage, PS::kBX>();
-  auto kern = k_pool_step<LAT, S, C, PS::kStage, PS::kBX>;
+  auto kern = k_pool_step<LAT, S, C, PS::kStage, PS::kBX, PS::kMinB>;
   if (smem && cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
     return 0;
   int dev = 0, sms = 0, per_sm = 0;
