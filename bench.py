@@ -38,12 +38,12 @@ L2_BYTES = 129 * 1024 * 1024
 # FP64 paths are bound by GB300's FP64 pipe, not by HBM.  Peak: 152 SMs x 2
 # FP64 instructions per clock x 2 flop (FMA) x 2.07 GHz = 1.259 TFLOP/s
 # (the GPU's nominal 1.25 TFLOP/s FP64 rate).  Flops per cell update of the
-# FP64 step from ncu's SASS counters of the plain one-thread-per-cell kernel
-# (profiles/step_d2q37_f64_1024.md, profiles/step_d3q107_f64_64.md):
-# D2Q37 299 DFMA + 175 DADD + 95 DMUL per cell = 868 flop;
-# D3Q107 786 DFMA + 511 DADD + 152 DMUL per cell = 2235 flop.
+# FP64 step from ncu's SASS counters (profiles/step_d2q37_f64_1024.md,
+# profiles/step_d3q107_f64_64.md):
+# D2Q37 294 DFMA + 148 DADD + 95 DMUL per cell = 831 flop;
+# D3Q107 761 DFMA + 428 DADD + 177 DMUL per cell = 2127 flop.
 FP64_PEAK_GFLOPS = 152 * 2 * 2 * 2.07
-FP64_FLOPS_PER_CELL = {0: 868, 1: 2235}
+FP64_FLOPS_PER_CELL = {0: 831, 1: 2127}
 
 WORKLOADS = {
     # name: lattice, prec, shape, gamma, tau_f, tau_g, steps per solve, fields
@@ -441,12 +441,15 @@ def run_ours(args, wl):
     word = {"f64": 8, "f32": 4, "f32_s16f": 2, "f32_s16bf": 2}[wl["prec"]]
     cells_per_s = N / step_kernel_s
     Q = 37 if wl["lattice"] == 0 else 107
-    bytes_per_cell = 2 * Q * 2 * word
+    # the two-step kernel reads and writes each population once per two updates
+    per_launch = steps_per_launch(wl, shape)
+    bytes_per_cell = 2 * Q * 2 * word / per_launch
     peak, peak_kind = measured_peaks()
     achieved = N * bytes_per_cell / step_kernel_s / 1e9
-    kname = "k_step_fd" if wl.get("scheme") == "fd" else "k_step"
+    kname = "k_step_fd" if wl.get("scheme") == "fd" else "k_step_pair" if per_launch == 2 else "k_step"
     key = f"{kname}_{'d2q37' if wl['lattice'] == 0 else 'd3q107'}_{wl['prec']}_{'x'.join(map(str, shape))}"
-    traffic = recorded_traffic(key)
+    traffic = recorded_traffic(key)  # of a launch; reported per step, as the other figures
+    traffic = traffic / per_launch if traffic else None
 
     cpu = None
     if world == 1 and not args.no_cpu_baseline:
@@ -467,14 +470,14 @@ def run_ours(args, wl):
                    **({"fd_kernel": args.fd_kernel} if wl.get("scheme") == "fd" else {})},
         "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                      "frac": achieved / peak, "traffic": traffic,
-                     "kernel": key, "bytes_per_cell_update": bytes_per_cell,
+                     "kernel": key, "bytes_per_cell_update": bytes_per_cell, "steps_per_launch": per_launch,
                      "step_kernel_us": step_kernel_s * 1e6, "peak_kind": peak_kind,
                      "shape": {"stage": tuned["stage"], "block": tuned["block"], "index": tuned["index"]}},
         "e2e": {"value": e2e_mlups, "unit": "MLUPS", "h2d_bytes_per_step": (2 + D) * N * 8,
                 "d2h_bytes_per_step": (2 + D) * N * 8,
                 "note": "per bench step = one solve through lbm_init (pinned host fields) + lbm_step + "
                         "lbm_moments (pinned host outputs)"},
-        "gpu_launches": args.steps * (S * step_launches(wl, shape) + 2),
+        "gpu_launches": args.steps * (-(-S // per_launch) * step_launches(wl, shape) + 2),
         "clocks": clk,
         "cpu_baseline": cpu,
     }
@@ -527,6 +530,18 @@ def step_launches(wl, shape):
     E = {"f64": 8, "f32": 4, "f32_s16f": 4, "f32_s16bf": 4}[wl["prec"]]
     border = ny * nz - (ny - 6) * (nz - 6)
     return 2 if ny >= 7 and nz >= 7 and nx * ny * nz * E < 2 ** 32 and border <= 65535 else 1
+
+
+def steps_per_launch(wl, shape):
+    """Lattice steps per launch of lbm_step: two on D2Q37 FP32 grids that the
+    two-step kernel's strips of 122 columns and bands of rows fill well
+    (pair_grid in launch_impl.cuh, with the GPU's 152 SMs), else one."""
+    if len(shape) != 2 or wl["prec"] != "f32" or wl.get("scheme") == "fd":
+        return 1
+    nx, ny = shape
+    strips = -(-nx // 122)
+    cost = min(-(-strips * nb // 152) * (-(-ny // nb) + 7) for nb in range(1, min(ny, 512) + 1))
+    return 2 if nx * ny / (122 * 152 * cost) >= 0.6 else 1
 
 
 def roofline_of(wl, N, step_s):
