@@ -33,6 +33,7 @@
 #include <type_traits>
 
 #include "lattice.h"
+#include "pair_order.h"
 
 namespace lbm {
 
@@ -1453,7 +1454,8 @@ __global__ void __launch_bounds__(BX, MINB) k_step_mirror(const S* __restrict__ 
 //   Order: A's groups take the even and the odd rows, B's likewise, so that
 // one group's loads overlap the other's arithmetic (16 warps of 128
 // registers).  A stores row t once B has pulled row t - 8 of the band, B
-// pulls row q once A's rows up to q + 6 are stored; both wait on mbarriers.
+// pulls row q once A's rows up to q + 6 are stored; both wait on mbarriers, by
+// the rules of pair_order.h, which says why no wait can miss its phase.
 //   A's columns are the strip's w and 3 on each side, its rows the band's
 // and 3 above and below, each mapped to a grid cell by the axis' rule
 // (wrapped, or the edge cell's again at a zero-gradient end), so B pulls
@@ -1531,7 +1533,7 @@ __global__ void __launch_bounds__(4 * kPairW, 1) k_step_pair(const float* __rest
   using L = Lat<0>;
   using S = float;
   using C = float;
-  constexpr int Q = L::Q, W = kPairW, NPL = 2, NB = 8;
+  constexpr int Q = L::Q, W = kPairW, NPL = 2, NB = kPairBars;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ unsigned long long stored[NB], pulled[NB];  // A's row t, B's row q (mod NB)
   wait_for_previous_kernel();
@@ -1605,9 +1607,8 @@ __global__ void __launch_bounds__(4 * kPairW, 1) k_step_pair(const float* __rest
         if (!(isfinite(drho) && isfinite(dT))) atomicOr(a.flag, 1u);
         eq_coeffs<0, C>(drho, u, dT, a, k);
       }
-      // the rows this one replaces were last pulled by B's row t - 8; the band's
-      // first rows replace none, but must not overtake the other group's
-      if (t >= 8 ? !wait(pulled, t - 8) : t >= 3 && !wait(stored, t - 3)) return;
+      if (pair_a_pulled(t) >= 0 && !wait(pulled, pair_a_pulled(t))) return;
+      if (pair_a_stored(t) >= 0 && !wait(stored, pair_a_stored(t))) return;
       if (active)
         relax_put_k<0, S, C, false, 0, Q>(getg, geth, [](auto) { return ConvGH<C>{C(0), C(0)}; }, a, k,
                                           [&](auto I, C gn, C hn) {
@@ -1624,10 +1625,9 @@ __global__ void __launch_bounds__(4 * kPairW, 1) k_step_pair(const float* __rest
     const bool active = j < w && x0 + j < nx;
     // B's row q pulls direction i from A's row q + 3 - c_y
     static_for<7>([&](auto K) { slot[decltype(K)::value] = slot_of(K, group - 2 + 6 - decltype(K)::value); });
-    int seen = 0;  // A's rows known to be stored
     for (int q = group - 2; q < rows; q += 2) {
-      for (; seen <= q + 6; ++seen)
-        if (!wait(stored, seen)) return;
+      for (int n = pair_b_begin(q); n <= pair_b_end(q); ++n)
+        if (!wait(stored, n)) return;
       C g[Q], h[Q];
       static_for<Q>([&](auto I) {
         constexpr int i = decltype(I)::value, kc = L::cy(i) + 3;
