@@ -1930,27 +1930,35 @@ __global__ void k_moments(const S* __restrict__ src, double* __restrict__ rho, d
 // long before HBM: a term-by-term FP64 sum takes about 5 FP64 instructions
 // per direction (185 per D2Q37 cell, plus a conversion per value), and HBM
 // delivers a cell's FP32 values every 26.  So FP32 and 16-bit storage sum on
-// the FP32 pipe first, without losing a bit of a term: every accumulator is
-// an unevaluated sum hi + lo, each addition to hi keeps its rounding error
-// (Knuth's two-sum) and adds it to lo.  There is one accumulator per
-// velocity group (for mass and kinetic energy), one for h, and one per axis
-// and |c_a| (momentum); after at most kTotalsRun cells of a thread they are
-// added up in FP64 with the factors c, |c|^2.  lo's own rounding is 2^-24 of
-// lo, at most (terms) 2^-48 of hi; against exact sums of the stored values
-// the totals are as near as the term-by-term FP64 sum's (2e-16 of the mass
-// and of the energy).  A run whose hi is not finite (values that are
-// infinite or NaN, or too large to sum in FP32) is summed again term by term
-// in FP64.  FP64 storage sums its pairs and groups in FP64.
-//   Measured, one lbm_conserved call (about 50 us of it the host's wait):
-// D2Q37 FP32 2048^2 2133 -> 281 us, FP16 storage 2075 -> 225 us, D3Q107 FP32
-// 128 x 128 x 127 3354 -> 396 us.  With 4-byte loads, each used as it
-// arrives, the first took 735 us: too few bytes in flight.
+// the FP32 pipe first: every accumulator is an unevaluated sum hi + lo, each
+// addition to hi keeps its rounding error (Knuth's two-sum) and adds it to
+// lo.  An addition to lo rounds too, by up to 2^-24 of lo, so over n terms
+// the sum could be off by some n^2 2^-49 of its largest partial sum -- unless
+// lo is exact.  It is where the terms are of like size: every error is a
+// multiple of the last place of the smallest term and lo stays below 2^24 of
+// those while n max|x| < 2^24 min|x| or so.  Hence the order of the sums: the
+// directions of one velocity group, whose weights are equal, over up to
+// kTotalsRun cells of a thread, with accumulators for g, h and, per axis, each
+// |c_a|; then they are added up in FP64 with the factors c, |c|^2 (34 sums
+// for D2Q37, 53 for D3Q107, 4 FP64 instructions each).  Sums of h over all groups in one
+// accumulator were off by up to 1e-12 on uniform fields, where every thread
+// makes the same error; these are within 2e-15 there and on random fields
+// (tests/test_gpu_totals_exact.py), as term-by-term FP64 sums are.  A run
+// with a sum that is not finite (values that are infinite or NaN, or too
+// large to sum in FP32) is summed again term by term in FP64.  FP64 storage
+// sums its pairs and groups in FP64.
+//   Measured, k_conserve_partial alone, one accumulator for h -> these: D2Q37
+// FP32 2048^2 247 -> 211 us, FP16 storage 186 -> 182, D3Q107 FP32 128 x 128 x
+// 127 353 -> 377, FP16 storage 379 -> 336; D2Q37 FP32 300^2 20.6 -> 24.1 (four
+// cells per thread carry all 34 FP64 additions).  Without the next group's
+// first loads issued before the present group's FP64 additions 261, 218, 398,
+// 370 us; runs of 16 cells 232, 199, 378, 341.
 // ---------------------------------------------------------------------------
 constexpr int kRedThreads = 256;
 constexpr int kRedMaxBlocks = 1024;  // partials an instance has room for
 constexpr int kRedBlocks = 6 * 152;    // blocks of a large grid: whole waves of 2, 3 or 6 blocks on each of 152 SMs
 constexpr int kRedVals = 5;  // mass, momentum[3], energy
-constexpr int kTotalsRun = 16;
+constexpr int kTotalsRun = 32;
 
 __device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll
@@ -1969,6 +1977,34 @@ __device__ __forceinline__ void two_sum(f32x2& hi, f32x2& lo, f32x2 x) {
   lo = add_f32x2(lo, add_f32x2(sub_f32x2(hi, sub_f32x2(s, b)), sub_f32x2(x, b)));
   hi = s;
 }
+
+// a velocity group in the totals: its directions [first, first + count), and
+// the values that |c_a| takes in it (one or two besides 0)
+template <int LAT, int GRP>
+struct TotalsGroup {
+  using L = Lat<LAT>;
+  static constexpr int g = GRP;
+  static constexpr int c2 = (LAT == 0 ? kD2Q37 : kD3Q107).c2[GRP];
+  static constexpr int count = (LAT == 0 ? kD2Q37 : kD3Q107).members[GRP];
+  static constexpr int begin() {
+    int i = 0;
+    while (L::grp(i) != GRP) ++i;
+    return i;
+  }
+  static constexpr int first = begin();
+  __host__ __device__ static constexpr int value(int k) {  // the (k + 1)-th of them in order of size, or 0
+    for (int v = 1; v <= 3; ++v)
+      for (int a = 0; a < L::D; ++a)
+        if ((LAT == 0 ? kD2Q37 : kD3Q107).rep[GRP][a] == v) {
+          if (k-- == 0) return v;
+          break;
+        }
+    return 0;
+  }
+  static constexpr int batch = count % 4 == 0 ? 4 : (count % 3 == 0 ? 3 : 1);  // directions per batch of loads
+  static constexpr int speeds = value(1) != 0 ? 2 : 1;
+  __host__ __device__ static constexpr int speed(int v) { return v == value(0) ? 0 : 1; }
+};
 
 // the totals of the cells begin, begin + stride, ... below end, every term
 // added in FP64
@@ -2037,59 +2073,69 @@ __device__ __forceinline__ void add_totals(const S* __restrict__ src, long long 
     // flight); the cells' values are summed in the two halves of f32x2
     constexpr int V = VEC;
     using W = typename std::conditional<V == 4, uint4, unsigned>::type;
-    auto value = [](unsigned w) { return __uint_as_float(w); };
+    constexpr int NPL = IsS16<S>::value ? 1 : 2;
     while (begin < end) {
       const long long first = begin;
-      f32x2 hi[G], lo[G], jhi[D][3], jlo[D][3], hhi = 0, hlo = 0;
+      begin = min(end, first + (kTotalsRun / V) * stride);
+      double part[kRedVals] = {0.0, 0.0, 0.0, 0.0, 0.0};
+      bool fine = true;
+      // the batch of loads that is issued while the one before is summed, also
+      // from one quad of cells and from one group to the next
+      W next[4][NPL];
+      auto fetch = [&](auto K, auto M, long long cell) {
+        using R = TotalsGroup<LAT, decltype(K)::value>;
+        static_for<R::batch>([&](auto J) {
+          constexpr int i = R::first + decltype(M)::value * R::batch + decltype(J)::value;
 #pragma unroll
-      for (int g = 0; g < G; ++g) hi[g] = lo[g] = 0ull;
-#pragma unroll
-      for (int a = 0; a < D; ++a)
-#pragma unroll
-        for (int c = 0; c < 3; ++c) jhi[a][c] = jlo[a][c] = 0ull;
-      auto add = [&](auto I, f32x2 g, f32x2 h) {
-        constexpr int i = decltype(I)::value;
-        if constexpr (IsS16<S>::value) {  // the 16-bit codec in FP32, as the step evaluates it
-          float a0, a1;
-          unpack_f32x2(g, a0, a1);
-          g = pack_f32x2(__fmul_rn(a0, af.gref[L::grp(i)]), __fmul_rn(a1, af.gref[L::grp(i)]));
-          unpack_f32x2(h, a0, a1);
-          h = pack_f32x2(__fmul_rn(a0, af.hscale[L::grp(i)]), __fmul_rn(a1, af.hscale[L::grp(i)]));
-        }
-        two_sum(hi[L::grp(i)], lo[L::grp(i)], g);
-        two_sum(hhi, hlo, h);
-        auto axis = [&](int a, int c) {
-          if (c > 0) two_sum(jhi[a][c - 1], jlo[a][c - 1], g);
-          if (c < 0) two_sum(jhi[a][-c - 1], jlo[a][-c - 1], neg_f32x2(g));
-        };
-        axis(0, L::cx(i));
-        axis(1, L::cy(i));
-        if constexpr (D == 3) axis(2, L::cz(i));
+          for (int q = 0; q < NPL; ++q)
+            next[decltype(J)::value][q] = ld_again(reinterpret_cast<const W*>(
+                reinterpret_cast<const unsigned*>(src) + ((size_t)(q * Q + i) * ps + cell)));
+        });
       };
-#pragma unroll 1
-      for (int k = 0; k < kTotalsRun / V && begin < end; ++k, begin += stride) {
-        // the next directions' loads are issued before the present ones are summed
-        constexpr int B = V == 4 ? 3 : 8, NB = (Q + B - 1) / B, NPL = IsS16<S>::value ? 1 : 2;
-        W buf[2][B][NPL];
-        auto fetch = [&](auto K) {
-          static_for<B>([&](auto J) {
-            constexpr int i = decltype(K)::value * B + decltype(J)::value;
-            if constexpr (i < Q) {
+      fetch(std::integral_constant<int, 0>{}, std::integral_constant<int, 0>{}, first);
+      static_for<G>([&](auto K) {
+        using R = TotalsGroup<LAT, decltype(K)::value>;
+        constexpr int NB = R::count / R::batch;
+        f32x2 ghi = 0ull, glo = 0ull, hhi = 0ull, hlo = 0ull, jhi[D][R::speeds], jlo[D][R::speeds];
 #pragma unroll
-              for (int q = 0; q < NPL; ++q)
-                buf[decltype(K)::value % 2][decltype(J)::value][q] =
-                    ld_again(reinterpret_cast<const W*>(reinterpret_cast<const unsigned*>(src) + ((size_t)(q * Q + i) * ps + begin)));
-            }
-          });
+        for (int a = 0; a < D; ++a)
+#pragma unroll
+          for (int c = 0; c < R::speeds; ++c) jhi[a][c] = jlo[a][c] = 0ull;
+        auto add = [&](auto I, f32x2 g, f32x2 h) {
+          constexpr int i = decltype(I)::value;
+          if constexpr (IsS16<S>::value) {  // the 16-bit codec in FP32, as the step evaluates it
+            float a0, a1;
+            unpack_f32x2(g, a0, a1);
+            g = pack_f32x2(__fmul_rn(a0, af.gref[R::g]), __fmul_rn(a1, af.gref[R::g]));
+            unpack_f32x2(h, a0, a1);
+            h = pack_f32x2(__fmul_rn(a0, af.hscale[R::g]), __fmul_rn(a1, af.hscale[R::g]));
+          }
+          two_sum(ghi, glo, g);
+          two_sum(hhi, hlo, h);
+          auto axis = [&](int a, int c) {
+            if (c > 0) two_sum(jhi[a][R::speed(c)], jlo[a][R::speed(c)], g);
+            if (c < 0) two_sum(jhi[a][R::speed(-c)], jlo[a][R::speed(-c)], neg_f32x2(g));
+          };
+          axis(0, L::cx(i));
+          axis(1, L::cy(i));
+          if constexpr (D == 3) axis(2, L::cz(i));
         };
-        fetch(std::integral_constant<int, 0>{});
-        static_for<NB>([&](auto K) {
-          constexpr int kk = decltype(K)::value;
-          if constexpr (kk + 1 < NB) fetch(std::integral_constant<int, kk + 1>{});
-          static_for<B>([&](auto J) {
-            constexpr int i = kk * B + decltype(J)::value;
-            if constexpr (i < Q) {
-              const W(&w)[NPL] = buf[kk % 2][decltype(J)::value];
+#pragma unroll 1
+        for (long long cell = first; cell < begin; cell += stride) {
+          static_for<NB>([&](auto M) {
+            constexpr int m = decltype(M)::value;
+            W now[R::batch][NPL];
+            static_for<R::batch>([&](auto J) {
+#pragma unroll
+              for (int q = 0; q < NPL; ++q) now[decltype(J)::value][q] = next[decltype(J)::value][q];
+            });
+            if constexpr (m + 1 < NB) fetch(K, std::integral_constant<int, m + 1>{}, cell);
+            else if (cell + stride < begin) fetch(K, std::integral_constant<int, 0>{}, cell + stride);
+            else if constexpr (R::g + 1 < G)
+              fetch(std::integral_constant<int, R::g + 1>{}, std::integral_constant<int, 0>{}, first);
+            static_for<R::batch>([&](auto J) {
+              constexpr int i = R::first + m * R::batch + decltype(J)::value;
+              const W(&w)[NPL] = now[decltype(J)::value];
               auto two = [&](unsigned g0, unsigned g1, unsigned h0, unsigned h1) {
                 if constexpr (IsS16<S>::value) {
                   float ga, ha, gb, hb;
@@ -2097,7 +2143,8 @@ __device__ __forceinline__ void add_totals(const S* __restrict__ src, long long 
                   unpack16<S>(g1, gb, hb);
                   add(std::integral_constant<int, i>{}, pack_f32x2(ga, gb), pack_f32x2(ha, hb));
                 } else {
-                  add(std::integral_constant<int, i>{}, pack_f32x2(value(g0), value(g1)), pack_f32x2(value(h0), value(h1)));
+                  add(std::integral_constant<int, i>{}, pack_f32x2(__uint_as_float(g0), __uint_as_float(g1)),
+                      pack_f32x2(__uint_as_float(h0), __uint_as_float(h1)));
                 }
               };
               if constexpr (V == 4) {
@@ -2106,33 +2153,26 @@ __device__ __forceinline__ void add_totals(const S* __restrict__ src, long long 
               } else {
                 two(w[0], 0u, w[NPL - 1], 0u);
               }
-            }
+            });
           });
-        });
-      }
-      bool fine = true;
-      auto total = [&](f32x2 h2, f32x2 l2) {
-        float h0, h1, l0, l1;
-        unpack_f32x2(h2, h0, h1);
-        unpack_f32x2(l2, l0, l1);
-        fine = fine && isfinite(h0) && isfinite(h1);
-        return (double(h0) + double(l0)) + (double(h1) + double(l1));
-      };
-      double part[kRedVals] = {0.0, 0.0, 0.0, 0.0, total(hhi, hlo)};
-      static_for<G>([&](auto K) {
-        constexpr int g = decltype(K)::value;
-        constexpr int c2 = (LAT == 0 ? kD2Q37 : kD3Q107).c2[g];
-        const double m = total(hi[g], lo[g]);
+        }
+        auto total = [&](f32x2 h2, f32x2 l2) {
+          float hi, x, lo, y;
+          unpack_f32x2(h2, hi, x);
+          unpack_f32x2(l2, lo, y);
+          two_sum(hi, lo, x);
+          lo = __fadd_rn(lo, y);
+          fine = fine && isfinite(hi) && isfinite(lo);
+          return double(hi) + double(lo);
+        };
+        const double m = total(ghi, glo);
         part[0] += m;
-        part[4] = fma(half_r2 * c2, m, part[4]);
+        part[4] += fma(half_r2 * R::c2, m, total(hhi, hlo));
+        static_for<D * R::speeds>([&](auto J) {
+          constexpr int a = decltype(J)::value / R::speeds, c = decltype(J)::value % R::speeds;
+          if constexpr (R::c2 != 0) part[1 + a] = fma(r * R::value(c), total(jhi[a][c], jlo[a][c]), part[1 + a]);
+        });
       });
-#pragma unroll
-      for (int a = 0; a < D; ++a) {
-        double j = 0.0;
-#pragma unroll
-        for (int c = 0; c < 3; ++c) j = fma(double(c + 1), total(jhi[a][c], jlo[a][c]), j);
-        part[1 + a] = r * j;
-      }
       if (!fine) {
 #pragma unroll
         for (int k = 0; k < kRedVals; ++k) part[k] = 0.0;
