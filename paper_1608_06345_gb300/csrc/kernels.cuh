@@ -1954,11 +1954,11 @@ __global__ void k_moments(const S* __restrict__ src, double* __restrict__ rho, d
 // first loads issued before the present group's FP64 additions 261, 218, 398,
 // 370 us; runs of 16 cells 232, 199, 378, 341.
 // ---------------------------------------------------------------------------
-constexpr int kRedThreads = 256;
 constexpr int kRedMaxBlocks = 1024;  // partials an instance has room for
-constexpr int kRedBlocks = 6 * 152;    // blocks of a large grid: whole waves of 2, 3 or 6 blocks on each of 152 SMs
 constexpr int kRedVals = 5;  // mass, momentum[3], energy
 constexpr int kTotalsRun = 32;
+template <class S>
+constexpr int totals_load() { return sizeof(S) == 8 ? 1 : 4; }  // cells per load
 
 __device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll
@@ -2203,22 +2203,22 @@ __device__ __forceinline__ void store_block_totals(const double (&acc)[kRedVals]
   }
 }
 
-template <int LAT, class S>
-__global__ void __launch_bounds__(kRedThreads, 2) k_conserve_partial(const S* __restrict__ src, long long N,
-                                                                   const Args<double> a, const Args<float> af,
-                                                                   double* __restrict__ partial) {
+template <int LAT, class S, int THREADS>
+__global__ void __launch_bounds__(THREADS, 512 / THREADS) k_conserve_partial(const S* __restrict__ src, long long N,
+                                                                             const Args<double> a, const Args<float> af,
+                                                                             double* __restrict__ partial) {
   double acc[kRedVals] = {0.0, 0.0, 0.0, 0.0, 0.0};
   // an instance's planes start on 256 bytes, so whole quads of cells can be
   // read at once; the last N mod 4 go to the first threads of the last block
-  constexpr int V = sizeof(S) == 8 ? 1 : 4;
+  constexpr int V = totals_load<S>();
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x, nt = (long long)gridDim.x * blockDim.x;
   const long long whole = N / V * V;
   add_totals<LAT, S, V>(src, a.ps, t * V, whole, nt * V, a.r, a.half_r2, af, acc);
   if constexpr (V > 1) {
     if (blockIdx.x == gridDim.x - 1)
-      add_totals<LAT, S, 1>(src, a.ps, whole + threadIdx.x, N, kRedThreads, a.r, a.half_r2, af, acc);
+      add_totals<LAT, S, 1>(src, a.ps, whole + threadIdx.x, N, THREADS, a.r, a.half_r2, af, acc);
   }
-  store_block_totals<kRedThreads>(acc, partial);
+  store_block_totals<THREADS>(acc, partial);
 }
 
 

@@ -2,6 +2,7 @@
 // one (lattice, storage type, compute type).
 #pragma once
 
+#include <algorithm>
 #include <atomic>
 
 #include "runtime.h"
@@ -532,10 +533,26 @@ cudaError_t launch_moments_t(const Instance* inst, const void* src, double* rho,
 }
 
 
+// Blocks of 64 threads while the grid takes no more of them than there are
+// partials (262144 cells at 4 cells per thread, 65536 in FP64), so that few
+// cells are spread over many SMs; else two blocks of 256 per SM, all resident
+// at once.  us per launch (k_conserve_partial), one block of 256 threads per
+// 256 cells up to 6 per SM -> this: D2Q37 FP32 4000 cells 20.7 -> 14.6, 300^2
+// 24.1 -> 18.6, 300000 cells 41.2 -> 32.9, 1024^2 96.5 -> 60.4, 2048^2 211 ->
+// 203; FP16 storage 600000 cells 63.7 -> 39.2, 2048^2 182 -> 179; FP64 40000 cells
+// 26.8 -> 18.6; D3Q107 FP32 48000 cells 40.0 -> 34.1, 128 x 128 x 127 377 ->
+// 297.
 template <int LAT, class S>
-cudaError_t launch_conserve_t(const Instance* inst, const void* src, double* partial, int nblocks) {
-  k_conserve_partial<LAT, S><<<nblocks, kRedThreads, 0, inst->stream>>>(static_cast<const S*>(src), inst->N,
-                                                                         inst->ad, inst->af, partial);
+cudaError_t launch_conserve_t(const Instance* inst, const void* src, double* partial, int* nblocks) {
+  constexpr int V = totals_load<S>();
+  const S* s = static_cast<const S*>(src);
+  if (inst->N <= 64LL * V * kRedMaxBlocks) {
+    *nblocks = (int)((inst->N + 64 * V - 1) / (64 * V));
+    k_conserve_partial<LAT, S, 64><<<*nblocks, 64, 0, inst->stream>>>(s, inst->N, inst->ad, inst->af, partial);
+  } else {
+    *nblocks = std::min(2 * device_sms(), kRedMaxBlocks);
+    k_conserve_partial<LAT, S, 256><<<*nblocks, 256, 0, inst->stream>>>(s, inst->N, inst->ad, inst->af, partial);
+  }
   return cudaGetLastError();
 }
 

@@ -149,15 +149,8 @@ cudaError_t launch_init(const Instance* I, void* dst, const double* rho, const d
 cudaError_t launch_moments(const Instance* I, const void* src, double* rho, double* u, double* T) {
   return launchers_of(I).moments(I, src, rho, u, T);
 }
-cudaError_t launch_conserve(const Instance* I, const void* src, double* partial, int nblocks) {
+cudaError_t launch_conserve(const Instance* I, const void* src, double* partial, int* nblocks) {
   return launchers_of(I).conserve(I, src, partial, nblocks);
-}
-
-int reduction_blocks(long long N) {
-  long long b = (N + kRedThreads - 1) / kRedThreads;
-  if (b > kRedBlocks) b = kRedBlocks;
-  if (b < 1) b = 1;
-  return (int)b;
 }
 
 // Enqueues the next step, or the next two in one launch where the instance
@@ -491,10 +484,10 @@ int lbm_moments(lbm_handle h, double* rho, double* u, double* T) {
 int lbm_conserved(lbm_handle h, double* out) {
   if (!h) return fail(LBM_EINVAL, "handle is NULL");
   if (!out) return fail(LBM_EINVAL, "out is NULL");
-  const int nb = reduction_blocks(h->N);
+  int nb = 0;
   cudaError_t e = cudaSuccess;
   if (h->N > 0) {
-    e = launch_conserve(h, h->buf[h->cur], h->red_partial, nb);
+    e = launch_conserve(h, h->buf[h->cur], h->red_partial, &nb);
     if (e == cudaSuccess) {
       k_conserve_final<<<1, 32 * kRedVals, 0, h->stream>>>(h->red_partial, nb, h->red_out);
       e = cudaGetLastError();

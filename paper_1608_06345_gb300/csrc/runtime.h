@@ -74,7 +74,7 @@ struct Launchers {
   cudaError_t (*step)(const Instance* inst, const void* src, void* dst);
   cudaError_t (*init)(const Instance* inst, void* dst, const double* rho, const double* u, const double* T);
   cudaError_t (*moments)(const Instance* inst, const void* src, double* rho, double* u, double* T);
-  cudaError_t (*conserve)(const Instance* inst, const void* src, double* partial, int nblocks);
+  cudaError_t (*conserve)(const Instance* inst, const void* src, double* partial, int* nblocks);  // sets the partials written
   cudaError_t (*pool_step)(const PoolLaunch& pl);
   cudaError_t (*pool_advance)(const PoolLaunch& pl);
   int (*pool_grid)();

@@ -63,21 +63,23 @@ def test_uniform_planes_sum_exactly(lat, seed, N):
     check(got, v[: len(w)], v[len(w):], c, r, N)
 
 
-@pytest.mark.parametrize("lat,shape", [(0, (2048, 1900)), (1, (160, 160, 40))])
-def test_uniform_instance_sums_exactly(lat, shape):
-    """lbm_conserved, with runs of several quads of cells per thread."""
+# runs of several quads of cells per thread; then the cells at which the
+# blocks of 64 threads end (launch_conserve_t)
+@pytest.mark.parametrize("lat,shape,prec", [(0, (2048, 1900), 1), (1, (160, 160, 40), 1), (0, (1024, 256), 1),
+                                            (0, (5, 52429), 1), (0, (256, 256), 0), (0, (65537, 1), 0)])
+def test_uniform_instance_sums_exactly(lat, shape, prec):
     import torch
 
     from paper_1608_06345_gb300 import lbm
     c, w, r = lattice(lbm, lat)
     N, D = math.prod(shape), len(shape)
-    s = lbm.Solver(lat, GAMMA, 0.6, 0.7, shape, prec=lbm.LBM_F32, rho0=-1.0)
+    s = lbm.Solver(lat, GAMMA, 0.6, 0.7, shape, prec=prec, rho0=-1.0)
     u = torch.tensor([0.031, -0.017, 0.011][:D], dtype=torch.float64)[:, None].expand(-1, N).contiguous().cuda()
     s.init(torch.full((N,), 0.83, dtype=torch.float64, device="cuda"), u,
            torch.full((N,), 1.07, dtype=torch.float64, device="cuda"))
     got = s.conserved()
     ps = -(-N // 64) * 64
-    v = s.mem.view(torch.float32)[: 2 * len(w) * ps].reshape(-1, ps)[:, 0].double().cpu().numpy()
+    v = s.mem.view(torch.float64 if prec == 0 else torch.float32)[: 2 * len(w) * ps].reshape(-1, ps)[:, 0].double().cpu().numpy()
     s.close()
     check(got, v[: len(w)], v[len(w):], c, r, N)
 
