@@ -715,12 +715,12 @@ __device__ __forceinline__ void relax_store(GetG&& getg, GetH&& geth, Conv&& con
   relax_store_k<LAT, S, C, IDX32, FD, IB, IE>(getg, geth, conv, a, k, dst, ps, cell);
 }
 
-template <int LAT, class S, class C, bool IDX32, bool FD, class GetG, class GetH, class Conv>
-__device__ __forceinline__ void collide_store_impl(GetG&& getg, GetH&& geth, Conv&& conv, const Args<C>& a,
-                                                   S* __restrict__ dst, long long ps, unsigned cell) {
-  C drho, u[3], dT;
+// the moments of a cell as every one-thread-per-cell kernel sums them.  FP64:
+// in the four parts of k_step_split, so that the FP64 shapes, and the row and
+// the tile kernel of the finite-difference step, give the same bits
+template <int LAT, class S, class C, class GetG, class GetH>
+__device__ __forceinline__ void moments_cell(GetG&& getg, GetH&& geth, const Args<C>& a, C& drho, C (&u)[3], C& dT) {
   if constexpr (std::is_same<S, double>::value) {
-    // summed in the four parts of k_step_split, so that the FP64 shapes give the same bits
     C sum[5];
     static_for<4>([&](auto W) {
       constexpr int w = decltype(W)::value;
@@ -733,6 +733,13 @@ __device__ __forceinline__ void collide_store_impl(GetG&& getg, GetH&& geth, Con
   } else {
     moments_raw<LAT, C, IsS16<S>::value>(getg, geth, a, drho, u, dT);
   }
+}
+
+template <int LAT, class S, class C, bool IDX32, bool FD, class GetG, class GetH, class Conv>
+__device__ __forceinline__ void collide_store_impl(GetG&& getg, GetH&& geth, Conv&& conv, const Args<C>& a,
+                                                   S* __restrict__ dst, long long ps, unsigned cell) {
+  C drho, u[3], dT;
+  moments_cell<LAT, S, C>(getg, geth, a, drho, u, dT);
   if (!(isfinite(drho) && isfinite(dT))) atomicOr(a.flag, 1u);
   relax_store<LAT, S, C, IDX32, FD>(getg, geth, conv, a, drho, u, dT, dst, ps, cell);
 }
@@ -1779,7 +1786,7 @@ __global__ void __launch_bounds__(BX* BY* BZ, MINB) k_step_fd_tile(const S* __re
   C drho, u[3], dT;
   {
     C g, h;
-    moments_raw<LAT, C, IsS16<S>::value>(
+    moments_cell<LAT, S, C>(
         [&](auto I) { near(decltype(I)::value, cell, g, h); return g; },
         [&](auto I) { near(decltype(I)::value, cell, g, h); return h; }, a, drho, u, dT);
   }
