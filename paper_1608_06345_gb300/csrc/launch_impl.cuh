@@ -35,7 +35,9 @@ cudaError_t launch_next(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, 
   at[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
+  if (e != cudaSuccess) cudaGetLastError();  // the caller gets it; a later launch's check must not
+  return e;
 }
 
 inline int device_sms() {
