@@ -121,8 +121,11 @@ void fill_args(const Instance& I, Args<C>* a) {
   a->half_delta = (C)(0.5 * I.delta);
   a->omega_f = (C)(1.0 / I.tau_f);
   a->omega_g = (C)(1.0 / I.tau_g);
-  a->om1_f = (C)(1.0 - 1.0 / I.tau_f);
-  a->hd_fg = (C)(0.5 * I.delta * I.tau_f / I.tau_g);
+  // FP64 relaxation: 1 / tau_f of 1e-200 is nothing to any value of FP64, and
+  // below it the weights would be subnormal and delta tau_f infinite
+  const double tau = std::fmin(I.tau_f, 1e200);
+  a->om1_f = (C)(1.0 - 1.0 / tau);
+  a->hd_fg = (C)(0.5 * I.delta * tau / I.tau_g);
   a->rho0 = (C)I.rho0;
   a->T0 = (C)I.T0;
   a->t0 = (C)(I.T0 - 1.0);
@@ -130,7 +133,7 @@ void fill_args(const Instance& I, Args<C>* a) {
   reference_constants(I.table, I.delta, I.rho0, I.T0, gref, pref, hscale);
   for (int g = 0; g < 10; ++g) {
     a->wg[g] = (C)I.table.wg[g];
-    a->wf[g] = (C)(I.table.wg[g] / I.tau_f);
+    a->wf[g] = (C)(I.table.wg[g] / tau);
     a->x2g[g] = (C)I.table.x2g[g];
     a->gref[g] = (C)gref[g];
     a->pref[g] = (C)pref[g];
