@@ -1477,9 +1477,6 @@ __global__ void __launch_bounds__(BX, MINB) k_step_mirror(const S* __restrict__ 
 // thread in f32x2 arithmetic, 0.64 of the instructions but 8 warps, 1387;
 // rows brought to L2 ahead of the loads, 1400 - 1500.
 // ---------------------------------------------------------------------------
-constexpr int kPairW = 128;           // A's columns
-constexpr int kPairOut = kPairW - 6;  // columns a strip can hold
-
 struct PairRing {
   static constexpr int cy(int i) { return Lat<0>::cy(i); }
   static constexpr int depth(int k) { return k + 2; }  // rows kept of the directions with c_y = k - 3

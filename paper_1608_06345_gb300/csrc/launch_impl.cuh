@@ -40,18 +40,6 @@ cudaError_t launch_next(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, 
   return e;
 }
 
-inline int device_sms() {
-  static std::atomic<int> sms[64];
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev >= 64) return 152;
-  int n = sms[dev].load(std::memory_order_relaxed);
-  if (n == 0) {
-    if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 152;
-    sms[dev].store(n, std::memory_order_relaxed);
-  }
-  return n;
-}
-
 // dynamic shared memory of a step shape: none (STAGE 0, 6), h only (STAGE 3),
 // g and h (STAGE 1)
 template <int LAT, class S, int STAGE, int BX>
@@ -336,27 +324,6 @@ cudaError_t launch_step_shape(const Instance* inst, const void* src, void* dst, 
 // ---------------------------------------------------------------------------
 // two steps in one launch
 // ---------------------------------------------------------------------------
-// Strips of columns and bands of rows: one block fits an SM, a block's time
-// is that of its rows + 7 iterations, so take the number of bands with the
-// fewest iterations over all waves.  Returns the share of them that a grid of
-// full strips without those 7 would need.
-inline double pair_grid(const Instance* inst, int* strips, int* bands, int* width) {
-  const int nx = inst->n[0], ny = inst->n[1], sms = device_sms();
-  *strips = (nx + kPairOut - 1) / kPairOut;
-  *width = (nx + *strips - 1) / *strips;
-  long long best = -1;
-  *bands = 1;
-  for (int nb = 1; nb <= ny && nb <= 512; ++nb) {
-    const long long waves = ((long long)*strips * nb + sms - 1) / sms;
-    const long long cost = waves * ((ny + nb - 1) / nb + 7);
-    if (best < 0 || cost < best) {
-      best = cost;
-      *bands = nb;
-    }
-  }
-  return (double)inst->N / ((double)kPairOut * sms * (double)best);
-}
-
 // Whether two steps per launch are the faster way.  Measured against the
 // share of pair_grid: 0.44 (384^2) 0.79 of the single step's speed, 0.57
 // (512^2) 1.03, 0.60 (100 x 6000) 1.18, 0.72 (768^2) 1.15, 0.80 (1024^2)
@@ -364,8 +331,7 @@ inline double pair_grid(const Instance* inst, int* strips, int* bands, int* widt
 template <int LAT, class S, class C>
 bool has_pair_t(const Instance* inst) {
   if constexpr (LAT == 0 && std::is_same<S, float>::value) {
-    int strips, bands, width;
-    return pair_grid(inst, &strips, &bands, &width) >= 0.6;
+    return inst->pair.share >= 0.6;
   } else {
     return false;
   }
@@ -385,10 +351,9 @@ cudaError_t launch_pair_v(const Instance* inst, const void* src, void* dst, bool
     if (dev < 64) configured.fetch_or(1ull << dev, std::memory_order_release);
   }
   if (configure_only) return cudaSuccess;
-  int strips, bands, width;
-  pair_grid(inst, &strips, &bands, &width);
-  return launch_next(kern, dim3((unsigned)strips, (unsigned)bands), 4 * kPairW, smem, inst->stream,
-                     static_cast<const float*>(src), static_cast<float*>(dst), inst->af, width);
+  const PairGrid& g = inst->pair;
+  return launch_next(kern, dim3((unsigned)g.strips, (unsigned)g.bands), 4 * kPairW, smem, inst->stream,
+                     static_cast<const float*>(src), static_cast<float*>(dst), inst->af, g.width);
 }
 
 template <int LAT, class S, class C>

@@ -344,6 +344,7 @@ int lbm_create(lbm_handle* out, int lattice, double gamma, double tau_f, double 
   I->red_out = reinterpret_cast<double*>(tail + 256);
   I->red_partial = reinterpret_cast<double*>(tail + 512);
   I->cur = 0;
+  if (I->lattice == LBM_D2Q37 && I->prec == kF32) I->pair = pair_grid(I->n[0], I->n[1], device_sms());
   fill_instance_args(I);
   cudaError_t e = cudaMemsetAsync(tail, 0, kTailBytes, I->stream);
   if (e != cudaSuccess) {

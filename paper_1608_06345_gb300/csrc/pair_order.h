@@ -1,5 +1,5 @@
-// The waits of the two-step kernel (k_step_pair), as rules on row numbers, so
-// that the order can be checked on the host.
+// The two-step kernel's grid, and its waits as rules on row numbers, so that
+// both can be checked on the host.
 //
 // Two groups of warps (A) do the first step of the band's even and odd rows t
 // = 0 .. rows + 5, two groups (B) the second step of the even and odd rows q =
@@ -41,5 +41,38 @@ constexpr int pair_a_stored(int t) { return t < kPairBars ? t - 3 : -1; }
 // B may pull row q once A's rows pair_b_begin(q) .. pair_b_end(q) are stored
 constexpr int pair_b_begin(int q) { return q + 5; }
 constexpr int pair_b_end(int q) { return q + 6; }
+
+constexpr int kPairW = 128;           // A's columns
+constexpr int kPairOut = kPairW - 6;  // columns a strip can hold
+
+// The grid of the two-step kernel: strips of width columns by bands of rows.
+// share is that of the iterations which full strips without a band's 7 extra
+// iterations would need; 0 where there is no grid.
+struct PairGrid {
+  int strips, bands, width;
+  double share;
+};
+
+// One block fits an SM, and a block's time is that of its rows + 7 iterations,
+// so take the number of bands with the fewest iterations over all waves.  (512
+// candidates of two divisions each take a few microseconds of the host's time,
+// half of a small step's, so an instance does this once, when it is made.)
+inline PairGrid pair_grid(int nx, int ny, int sms) {
+  PairGrid g;
+  g.strips = (nx + kPairOut - 1) / kPairOut;
+  g.width = (nx + g.strips - 1) / g.strips;
+  g.bands = 1;
+  long long best = -1;
+  for (int nb = 1; nb <= ny && nb <= 512; ++nb) {
+    const long long waves = ((long long)g.strips * nb + sms - 1) / sms;
+    const long long cost = waves * ((ny + nb - 1) / nb + 7);
+    if (best < 0 || cost < best) {
+      best = cost;
+      g.bands = nb;
+    }
+  }
+  g.share = (double)((long long)nx * ny) / ((double)kPairOut * sms * (double)best);
+  return g;
+}
 
 }  // namespace lbm

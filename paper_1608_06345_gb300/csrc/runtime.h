@@ -6,11 +6,13 @@
 #include <stddef.h>
 #include <stdint.h>
 
+#include <atomic>
 #include <string>
 
 #include "../../include/lbm.h"
 #include "kernels.cuh"
 #include "lattice.h"
+#include "pair_order.h"
 
 namespace lbm {
 
@@ -50,10 +52,24 @@ struct Instance {
   int graph_shape;           // shape index the graph was captured with
   cudaGraphExec_t graph_exec;
   cudaGraph_t graph;
+  PairGrid pair;  // of a D2Q37 FP32 instance (lbm_create)
 };
 
 // Bytes of the tail region after the two buffers.
 constexpr size_t kTailBytes = 256 /*flag*/ + 256 /*red_out*/ + sizeof(double) * kRedMaxBlocks * kRedVals;
+
+// SMs of the current device
+inline int device_sms() {
+  static std::atomic<int> sms[64];
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev >= 64) return 152;
+  int n = sms[dev].load(std::memory_order_relaxed);
+  if (n == 0) {
+    if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 152;
+    sms[dev].store(n, std::memory_order_relaxed);
+  }
+  return n;
+}
 
 inline size_t round_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
