@@ -375,8 +375,8 @@ def run_ours(args, wl):
         tuned = {"index": -1, "stage": 0, "block": 128 if wl["lattice"] == 0 else 64}
     elif args.shape is not None:  # a fixed compiled shape instead of the autotuner's pick (profiling)
         lbm.lbm_set_shape(solver.h, args.shape)
-        st, bx = lbm.lbm_shape_info(wl["lattice"], prec, args.shape)
-        tuned = {"index": args.shape, "stage": st, "block": bx}
+        st, bx, per = lbm.lbm_step_info(solver.h)
+        tuned = {"index": args.shape, "stage": st, "block": bx, "steps_per_launch": per}
     else:
         tuned = autotune.tune(solver, reps=5, cache_path=None)
 
@@ -442,7 +442,7 @@ def run_ours(args, wl):
     cells_per_s = N / step_kernel_s
     Q = 37 if wl["lattice"] == 0 else 107
     # the two-step kernel reads and writes each population once per two updates
-    per_launch = steps_per_launch(wl, shape)
+    per_launch = tuned.get("steps_per_launch", 1)
     bytes_per_cell = 2 * Q * 2 * word / per_launch
     peak, peak_kind = measured_peaks()
     achieved = N * bytes_per_cell / step_kernel_s / 1e9
@@ -530,18 +530,6 @@ def step_launches(wl, shape):
     E = {"f64": 8, "f32": 4, "f32_s16f": 4, "f32_s16bf": 4}[wl["prec"]]
     border = ny * nz - (ny - 6) * (nz - 6)
     return 2 if ny >= 7 and nz >= 7 and nx * ny * nz * E < 2 ** 32 and border <= 65535 else 1
-
-
-def steps_per_launch(wl, shape):
-    """Lattice steps per launch of lbm_step: two on D2Q37 FP32 grids that the
-    two-step kernel's strips of 122 columns and bands of rows fill well
-    (pair_grid in launch_impl.cuh, with the GPU's 152 SMs), else one."""
-    if len(shape) != 2 or wl["prec"] != "f32" or wl.get("scheme") == "fd":
-        return 1
-    nx, ny = shape
-    strips = -(-nx // 122)
-    cost = min(-(-strips * nb // 152) * (-(-ny // nb) + 7) for nb in range(1, min(ny, 512) + 1))
-    return 2 if nx * ny / (122 * 152 * cost) >= 0.6 else 1
 
 
 def roofline_of(wl, N, step_s):

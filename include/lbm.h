@@ -124,12 +124,12 @@ int lbm_init_device(lbm_handle h, const double* rho, const double* u, const doub
  * stream.  Runs of at least twice the graph
  * length (lbm_set_graph_steps, default 64) replay a captured CUDA graph of
  * that many steps instead of launching each step, and large D2Q37 grids with
- * FP32 storage take two steps per launch; the arithmetic is the same, bit for
- * bit. */
+ * FP32 storage take two steps per launch while their shape is index 0
+ * (lbm_set_shape); the arithmetic is the same, bit for bit. */
 int lbm_step(lbm_handle h, long n);
 
 /* Steps per CUDA graph replay of lbm_step (even, 0..4096); 0 launches every
- * step separately (the plain one-launch-per-step path).  Execution control
+ * step separately (the plain one-launch-per-step path, whatever the shape).  Execution control
  * with no counterpart in the paper. */
 int lbm_set_graph_steps(lbm_handle h, int steps);
 
@@ -241,21 +241,33 @@ int lbm_conserved_noalloc(int lattice, int prec, double gamma, double rho0, doub
  * (stage 6) or half of them so and half in shared memory (stage 9), or two
  * lanes per cell, one for c and one for -c of every
  * (c, -c) pair, whose moment sums meet by warp shuffles (stage 8) -- and
- * the cells per thread block); index 0 is the default, which picks by the
- * grid's size among kernels that give the same bits.
- * lbm_shape_info describes candidate `index` (LBM_EINVAL past the end). */
+ * the cells per thread block).  Index 0 is the default, which picks by the
+ * grid's size among kernels that give the same bits, the two-step kernel
+ * (stage 10) among them; every other index is one kernel on every grid.
+ * lbm_shape_info describes candidate `index` (LBM_EINVAL past the end), index
+ * 0 by the single-step kernel of a large grid; lbm_step_info says what an
+ * instance runs. */
 int lbm_shape_info(int lattice, int prec, int index, int* stage, int* block);
 
-/* Select a candidate shape for this instance's steps. */
+/* Select a candidate shape for this instance's steps.  An index other than 0
+ * is the kernel of every step, one step per launch. */
 int lbm_set_shape(lbm_handle h, int index);
 
 /* Current shape index of the instance (-1 for NULL). */
 int lbm_get_shape(lbm_handle h);
 
+/* What lbm_step launches for the instance as it is: the kernel's stage and
+ * cells per block (two-step kernel: 10 and the columns a block works on) and
+ * the steps per launch, 1 or 2 (a single step that is left over runs alone).
+ * Any pointer may be NULL. */
+int lbm_step_info(lbm_handle h, int* stage, int* block, int* steps_per_launch);
+
 /* Time every candidate shape on this instance's own buffers (reps launches
  * each, CUDA events on its stream; the trials write only the idle buffer,
  * so the state does not change), select the fastest and return its index
- * and mean time per step in microseconds.  Synchronises. */
+ * and mean time per step in microseconds.  Index 0 is timed as lbm_step runs
+ * it, two steps per launch where it does so, and a candidate that is the same
+ * kernel as index 0's is not timed again.  Synchronises. */
 int lbm_autotune(lbm_handle h, int reps, int* best_index, double* best_us);
 
 /* ------------------------------------------------------------------------

@@ -15,7 +15,8 @@ DEFAULT_CACHE = os.path.join(os.path.expanduser("~"), ".cache", "paper_1608_0634
 def _key(solver):
     import torch
     props = torch.cuda.get_device_properties(torch.cuda.current_device())
-    return (f"lat{solver.lattice}-prec{solver.prec}-{'x'.join(map(str, solver.shape))}-"
+    # "v2": index 0 may be the two-step kernel, and others are other kernels than in records without it
+    return (f"v2-lat{solver.lattice}-prec{solver.prec}-{'x'.join(map(str, solver.shape))}-"
             f"sm{props.multi_processor_count}")
 
 
@@ -29,15 +30,16 @@ def _load(path):
 
 def tune(solver, reps=5, cache_path=DEFAULT_CACHE, refresh=False):
     """Select the fastest shape for `solver` (an lbm.Solver).  Returns a dict
-    with the chosen index, its (stage, block) and the time per step."""
+    with the chosen index, the (stage, block) and steps per launch that lbm_step
+    then runs, and the time per step."""
     key = _key(solver)
     cache = _load(cache_path) if cache_path else {}
     if not refresh and key in cache:
         lbm.lbm_set_shape(solver.h, cache[key]["index"])
         return dict(cache[key], cached=True)
     index, us = lbm.lbm_autotune(solver.h, reps)
-    stage, block = lbm.lbm_shape_info(solver.lattice, solver.prec, index)
-    rec = {"index": index, "stage": stage, "block": block, "us_per_step": us}
+    stage, block, steps = lbm.lbm_step_info(solver.h)
+    rec = {"index": index, "stage": stage, "block": block, "steps_per_launch": steps, "us_per_step": us}
     if cache_path:
         cache[key] = rec
         os.makedirs(os.path.dirname(cache_path), exist_ok=True)

@@ -190,13 +190,16 @@ cudaError_t launch_step_mirror(const Instance* inst, const void* src, void* dst,
 }
 
 // Candidate shapes of the step per (lattice, storage), tried by the
-// autotuner; index 0 is the default.  (stage, cells per block, minimum
-// resident blocks per SM requested from the compiler, which caps registers):
+// autotuner: (stage, cells per block, minimum resident blocks per SM requested
+// from the compiler, which caps registers).  Index 0 picks by the grid's size
+// among shapes of one rounding (pick), and takes two steps per launch where
+// that is the faster way (has_pair_t); its row is what a large grid takes.
+// The other indices are the kernel that their row names, on every grid:
 //   D2Q37 FP32:        (0,128,4) (0,256,2) (0,64,8) (0,128,1)
 //   D2Q37 16-bit:      (6,128,8) (6,128,7) (6,128,6) (6,256,3) (0,128,4) (0,64,8)
 //   D2Q37 FP64:        (0,128,1) (0,256,1) (0,64,1)  (4,32,4)  (7,32,4)
-//   D3Q107 FP32:       (3,64,6)  (3,64,6)  (3,32,12) (4,32,6)  (8,32,8)  (8,64,4)  (3,128,3)
-//   D3Q107 FP64:       (1,64,1)  (4,32,3)  (4,32,2)  (7,32,3)
+//   D3Q107 FP32:       (3,128,3) (3,64,6)  (3,32,12) (4,32,6)  (8,32,8)  (8,64,4)  (3,128,3)
+//   D3Q107 FP64:       (7,32,3)  (4,32,3)  (4,32,2)  (7,32,3)
 //   D3Q107 16-bit:     (6,64,6)  (9,256,2) (6,32,12) (4,32,6)  (8,32,10) (8,32,12) (6,128,3)
 // Stage 4 is the velocity-split step: 4 warps per block of 32 cells; stage 7
 // the same with the per-cell coefficients formed once by warp 0 and shared.
@@ -205,25 +208,54 @@ cudaError_t launch_step_mirror(const Instance* inst, const void* src, void* dst,
 // pairs packed in registers and stages the other half in shared memory.  In FP32 the
 // moments of stages 4, 7 and 8 are summed in another order, so their results
 // differ from the other shapes' by rounding; in FP64 every shape sums them in
-// the order of stage 4.  Index 0 picks by the grid's size among shapes of one
-// rounding (launch_step_shape), the one the batched pool has, so a pooled
-// instance's result is bitwise that of a lone one.
+// the order of stage 4.  Index 0's shapes have the rounding of the batched
+// pool's, so a pooled instance's result is bitwise that of a lone one.
+struct ShapeRow {
+  int stage, bx, minb;
+  bool operator==(const ShapeRow& o) const { return stage == o.stage && bx == o.bx && minb == o.minb; }
+};
+
 template <int LAT, class S>
 struct StepShapes {
   static constexpr int count =
       (LAT == 0) ? (sizeof(S) == 8 ? 5 : (sizeof(S) == 2 ? 6 : 4)) : (sizeof(S) == 8 ? 4 : 7);
-  static void get(int k, int* stage, int* bx, int* minb) {
-    static const int s2[4][3] = {{0, 128, 4}, {0, 256, 2}, {0, 64, 8}, {0, 128, 1}};
-    static const int s2h[6][3] = {{6, 128, 8}, {6, 128, 7}, {6, 128, 6}, {6, 256, 3}, {0, 128, 4}, {0, 64, 8}};
-    static const int s2d[5][3] = {{0, 128, 1}, {0, 256, 1}, {0, 64, 1}, {4, 32, 4}, {7, 32, 4}};
-    static const int s3f[7][3] = {{3, 64, 6}, {3, 64, 6}, {3, 32, 12}, {4, 32, 6}, {8, 32, 8}, {8, 64, 4}, {3, 128, 3}};
-    static const int s3d[4][3] = {{1, 64, 1}, {4, 32, 3}, {4, 32, 2}, {7, 32, 3}};
-    static const int s3h[7][3] = {{6, 64, 6}, {9, 256, 2}, {6, 32, 12}, {4, 32, 6}, {8, 32, 10}, {8, 32, 12}, {6, 128, 3}};
-    const int(*t)[3] = (LAT == 0) ? (sizeof(S) == 8 ? s2d : (sizeof(S) == 2 ? s2h : s2))
-                                  : (sizeof(S) == 4 ? s3f : (sizeof(S) == 8 ? s3d : s3h));
-    *stage = t[k][0];
-    *bx = t[k][1];
-    *minb = t[k][2];
+  static ShapeRow get(int k) {
+    static const ShapeRow s2[4] = {{0, 128, 4}, {0, 256, 2}, {0, 64, 8}, {0, 128, 1}};
+    static const ShapeRow s2h[6] = {{6, 128, 8}, {6, 128, 7}, {6, 128, 6}, {6, 256, 3}, {0, 128, 4}, {0, 64, 8}};
+    static const ShapeRow s2d[5] = {{0, 128, 1}, {0, 256, 1}, {0, 64, 1}, {4, 32, 4}, {7, 32, 4}};
+    static const ShapeRow s3f[7] = {{3, 128, 3}, {3, 64, 6}, {3, 32, 12}, {4, 32, 6}, {8, 32, 8}, {8, 64, 4}, {3, 128, 3}};
+    static const ShapeRow s3d[4] = {{7, 32, 3}, {4, 32, 3}, {4, 32, 2}, {7, 32, 3}};
+    static const ShapeRow s3h[7] = {{6, 64, 6}, {9, 256, 2}, {6, 32, 12}, {4, 32, 6}, {8, 32, 10}, {8, 32, 12}, {6, 128, 3}};
+    if (LAT == 0) return sizeof(S) == 8 ? s2d[k] : (sizeof(S) == 2 ? s2h[k] : s2[k]);
+    return sizeof(S) == 4 ? s3f[k] : (sizeof(S) == 8 ? s3d[k] : s3h[k]);
+  }
+  // the shape of one step of this instance with index k
+  static ShapeRow pick(const Instance* inst, int k) {
+    if (k != 0) return get(k);
+    if constexpr (LAT == 0 && sizeof(S) == 8) {
+      // a tube of a few blocks waits on one thread's chain of 560 FP64
+      // instructions per cell: split it while every SM has at most two
+      // 32-cell blocks (1000 x 4: 22.6 -> 9.4 us; 1000 x 16, 512 blocks:
+      // 22.8 us, split 30.2)
+      if ((long long)((inst->n[0] + 31) / 32) * inst->n[1] <= 2LL * device_sms()) return {4, 32, 4};
+    } else if constexpr (LAT == 1 && sizeof(S) < 8) {
+      // Blocks of 32 cells where they leave a seventh fewer threads past the
+      // row ends than blocks of 64 (us per step, 64 and 32 cells: FP32 32^3
+      // 14.6 / 7.7, 96^3 291 / 271).  The line leaves out rows of 193 cells,
+      // 256 and 224 threads, where the two are level: FP32 860 / 856, FP16
+      // storage 193 x 96 x 96 352 / 363, BF16 380 / 376.  Else 128 cells with
+      // FP32 storage where they pad no more (256 x 128 x 128 1221 -> 1190, 193
+      // x 130 x 97 860 -> 830, 112 x 96 x 80 286 -> 267).
+      auto padded = [&](int bx) { return (inst->n[0] + bx - 1) / bx * bx; };
+      constexpr int stage = sizeof(S) == 4 ? 3 : 6;
+      if (7 * padded(32) <= 6 * padded(64)) return {stage, 32, 12};
+      if (sizeof(S) == 4 && padded(128) == padded(64)) return {stage, 128, 3};
+      return {stage, 64, 6};
+    }
+    // D3Q107 FP64: the split with shared coefficients is the fastest at every
+    // size (one thread per cell with cp.async staging 1000 x 16 x 16 983 ->
+    // 779 us, 256 x 128 x 128 14.1 -> 12.7 ms, 32^3 273 -> 116)
+    return get(0);
   }
 };
 
@@ -231,107 +263,69 @@ template <int LAT, class S>
 int shape_count_t() { return StepShapes<LAT, S>::count; }
 
 template <int LAT, class S>
-void shape_get_t(int k, int* stage, int* bx) {
-  int minb = 1;
-  StepShapes<LAT, S>::get(k, stage, bx, &minb);
-}
-
-// The default D3Q107 shape of FP32 and 16-bit storage.  Blocks of 32 cells
-// where they leave a seventh fewer threads past the row ends than blocks of
-// 64 (us per step, 64 and 32 cells: FP32 32^3 14.6 / 7.7, 96^3 291 / 271; at
-// 193 cells, 224 threads for 256, 860 / 856); else 128 cells with FP32 storage
-// where they pad no more (256 x 128 x 128 1221 -> 1190, 193 x 130 x 97 860 ->
-// 830, 112 x 96 x 80 286 -> 267).
-template <int LAT, class S, class C, int STAGE>
-cudaError_t launch_default_3d(const Instance* inst, const void* src, void* dst, const Args<C>& a,
-                              bool configure_only) {
-  auto padded = [&](int bx) { return (inst->n[0] + bx - 1) / bx * bx; };
-  if (7 * padded(32) <= 6 * padded(64))
-    return launch_step_t<LAT, S, C, STAGE, 32, 12>(inst, src, dst, a, configure_only);
-  if constexpr (sizeof(S) == 4)
-    if (padded(128) == padded(64)) return launch_step_t<LAT, S, C, STAGE, 128, 3>(inst, src, dst, a, configure_only);
-  return launch_step_t<LAT, S, C, STAGE, 64, 6>(inst, src, dst, a, configure_only);
+void shape_get_t(const Instance* inst, int k, int* stage, int* bx, int* minb) {
+  const ShapeRow r = inst ? StepShapes<LAT, S>::pick(inst, k) : StepShapes<LAT, S>::get(k);
+  *stage = r.stage;
+  *bx = r.bx;
+  *minb = r.minb;
 }
 
 template <int LAT, class S, class C>
 cudaError_t launch_step_shape(const Instance* inst, const void* src, void* dst, bool configure_only = false) {
   const Args<C>& a = args_of<C>(inst);
-  const int k = inst->shape.index;
+  const ShapeRow r = StepShapes<LAT, S>::pick(inst, inst->shape.index);
   if constexpr (LAT == 0 && sizeof(S) == 8) {
-    switch (k) {
-      case 1: return launch_step_t<LAT, S, C, 0, 256>(inst, src, dst, a, configure_only);
-      case 2: return launch_step_t<LAT, S, C, 0, 64>(inst, src, dst, a, configure_only);
-      case 3: return launch_step_split<LAT, S, C, 4, 4>(inst, src, dst, a, configure_only);
-      case 4: return launch_step_split<LAT, S, C, 4, 4, true>(inst, src, dst, a, configure_only);
-      case 0:
-        // a tube of a few blocks waits on one thread's chain of 560 FP64
-        // instructions per cell: split it while every SM has at most two
-        // 32-cell blocks (1000 x 4: 22.6 -> 9.4 us; 1000 x 16, 512 blocks:
-        // 22.8 us, split 30.2)
-        if ((long long)((inst->n[0] + 31) / 32) * inst->n[1] <= 2LL * device_sms())
-          return launch_step_split<LAT, S, C, 4, 4>(inst, src, dst, a, configure_only);
-        return launch_step_t<LAT, S, C, 0, 128>(inst, src, dst, a, configure_only);
-      default: return launch_step_t<LAT, S, C, 0, 128>(inst, src, dst, a, configure_only);
-    }
+    if (r == ShapeRow{0, 128, 1}) return launch_step_t<LAT, S, C, 0, 128>(inst, src, dst, a, configure_only);
+    if (r == ShapeRow{0, 256, 1}) return launch_step_t<LAT, S, C, 0, 256>(inst, src, dst, a, configure_only);
+    if (r == ShapeRow{0, 64, 1}) return launch_step_t<LAT, S, C, 0, 64>(inst, src, dst, a, configure_only);
+    if (r == ShapeRow{4, 32, 4}) return launch_step_split<LAT, S, C, 4, 4>(inst, src, dst, a, configure_only);
+    if (r == ShapeRow{7, 32, 4}) return launch_step_split<LAT, S, C, 4, 4, true>(inst, src, dst, a, configure_only);
   } else if constexpr (LAT == 0 && sizeof(S) == 2) {
-    switch (k) {
-      case 1: return launch_step_t<LAT, S, C, 6, 128, 7>(inst, src, dst, a, configure_only);
-      case 2: return launch_step_t<LAT, S, C, 6, 128, 6>(inst, src, dst, a, configure_only);
-      case 3: return launch_step_t<LAT, S, C, 6, 256, 3>(inst, src, dst, a, configure_only);
-      case 4: return launch_step_t<LAT, S, C, 0, 128, 4>(inst, src, dst, a, configure_only);
-      case 5: return launch_step_t<LAT, S, C, 0, 64, 8>(inst, src, dst, a, configure_only);
-      default: return launch_step_t<LAT, S, C, 6, 128, 8>(inst, src, dst, a, configure_only);
-    }
+    if (r == ShapeRow{6, 128, 8}) return launch_step_t<LAT, S, C, 6, 128, 8>(inst, src, dst, a, configure_only);
+    if (r == ShapeRow{6, 128, 7}) return launch_step_t<LAT, S, C, 6, 128, 7>(inst, src, dst, a, configure_only);
+    if (r == ShapeRow{6, 128, 6}) return launch_step_t<LAT, S, C, 6, 128, 6>(inst, src, dst, a, configure_only);
+    if (r == ShapeRow{6, 256, 3}) return launch_step_t<LAT, S, C, 6, 256, 3>(inst, src, dst, a, configure_only);
+    if (r == ShapeRow{0, 128, 4}) return launch_step_t<LAT, S, C, 0, 128, 4>(inst, src, dst, a, configure_only);
+    if (r == ShapeRow{0, 64, 8}) return launch_step_t<LAT, S, C, 0, 64, 8>(inst, src, dst, a, configure_only);
   } else if constexpr (LAT == 0) {
-    switch (k) {
-      case 1: return launch_step_t<LAT, S, C, 0, 256, 2>(inst, src, dst, a, configure_only);
-      case 2: return launch_step_t<LAT, S, C, 0, 64, 8>(inst, src, dst, a, configure_only);
-      case 3: return launch_step_t<LAT, S, C, 0, 128, 1>(inst, src, dst, a, configure_only);
-      default: return launch_step_t<LAT, S, C, 0, 128, 4>(inst, src, dst, a, configure_only);
-    }
+    if (r == ShapeRow{0, 128, 4}) return launch_step_t<LAT, S, C, 0, 128, 4>(inst, src, dst, a, configure_only);
+    if (r == ShapeRow{0, 256, 2}) return launch_step_t<LAT, S, C, 0, 256, 2>(inst, src, dst, a, configure_only);
+    if (r == ShapeRow{0, 64, 8}) return launch_step_t<LAT, S, C, 0, 64, 8>(inst, src, dst, a, configure_only);
+    if (r == ShapeRow{0, 128, 1}) return launch_step_t<LAT, S, C, 0, 128, 1>(inst, src, dst, a, configure_only);
   } else if constexpr (sizeof(S) == 4) {
-    switch (k) {
-      case 1: return launch_step_t<LAT, S, C, 3, 64, 6>(inst, src, dst, a, configure_only);
-      case 2: return launch_step_t<LAT, S, C, 3, 32, 12>(inst, src, dst, a, configure_only);
-      case 3: return launch_step_split<LAT, S, C, 4, 6>(inst, src, dst, a, configure_only);
-      case 4: return launch_step_mirror<LAT, S, C, 64, 8, true>(inst, src, dst, a, configure_only);
-      case 5: return launch_step_mirror<LAT, S, C, 128, 4, true>(inst, src, dst, a, configure_only);
-      case 6: return launch_step_t<LAT, S, C, 3, 128, 3>(inst, src, dst, a, configure_only);
-      default: return launch_default_3d<LAT, S, C, 3>(inst, src, dst, a, configure_only);
-    }
+    if (r == ShapeRow{3, 128, 3}) return launch_step_t<LAT, S, C, 3, 128, 3>(inst, src, dst, a, configure_only);
+    if (r == ShapeRow{3, 64, 6}) return launch_step_t<LAT, S, C, 3, 64, 6>(inst, src, dst, a, configure_only);
+    if (r == ShapeRow{3, 32, 12}) return launch_step_t<LAT, S, C, 3, 32, 12>(inst, src, dst, a, configure_only);
+    if (r == ShapeRow{4, 32, 6}) return launch_step_split<LAT, S, C, 4, 6>(inst, src, dst, a, configure_only);
+    if (r == ShapeRow{8, 32, 8}) return launch_step_mirror<LAT, S, C, 64, 8, true>(inst, src, dst, a, configure_only);
+    if (r == ShapeRow{8, 64, 4}) return launch_step_mirror<LAT, S, C, 128, 4, true>(inst, src, dst, a, configure_only);
   } else if constexpr (sizeof(S) == 8) {
-    switch (k) {
-      case 1: return launch_step_split<LAT, S, C, 4, 3>(inst, src, dst, a, configure_only);
-      case 2: return launch_step_split<LAT, S, C, 4, 2>(inst, src, dst, a, configure_only);
-      case 3: return launch_step_split<LAT, S, C, 4, 3, true>(inst, src, dst, a, configure_only);
-      // the split with shared coefficients is the faster at every size: 1000 x
-      // 16 x 16 983 -> 779 us, 256 x 128 x 128 14.1 -> 12.7 ms, 32^3 273 -> 116
-      default: return launch_step_split<LAT, S, C, 4, 3, true>(inst, src, dst, a, configure_only);
-    }
+    if (r == ShapeRow{7, 32, 3}) return launch_step_split<LAT, S, C, 4, 3, true>(inst, src, dst, a, configure_only);
+    if (r == ShapeRow{4, 32, 3}) return launch_step_split<LAT, S, C, 4, 3>(inst, src, dst, a, configure_only);
+    if (r == ShapeRow{4, 32, 2}) return launch_step_split<LAT, S, C, 4, 2>(inst, src, dst, a, configure_only);
   } else {
-    switch (k) {
-      case 1: return launch_step_t<LAT, S, C, 9, 256, 2>(inst, src, dst, a, configure_only);
-      case 2: return launch_step_t<LAT, S, C, 6, 32, 12>(inst, src, dst, a, configure_only);
-      case 3: return launch_step_split<LAT, S, C, 4, 6>(inst, src, dst, a, configure_only);
-      case 4: return launch_step_mirror<LAT, S, C, 64, 10, false>(inst, src, dst, a, configure_only);
-      case 5: return launch_step_mirror<LAT, S, C, 64, 12, false>(inst, src, dst, a, configure_only);
-      case 6: return launch_step_t<LAT, S, C, 6, 128, 3>(inst, src, dst, a, configure_only);
-      default: return launch_default_3d<LAT, S, C, 6>(inst, src, dst, a, configure_only);
-    }
+    if (r == ShapeRow{6, 64, 6}) return launch_step_t<LAT, S, C, 6, 64, 6>(inst, src, dst, a, configure_only);
+    if (r == ShapeRow{9, 256, 2}) return launch_step_t<LAT, S, C, 9, 256, 2>(inst, src, dst, a, configure_only);
+    if (r == ShapeRow{6, 32, 12}) return launch_step_t<LAT, S, C, 6, 32, 12>(inst, src, dst, a, configure_only);
+    if (r == ShapeRow{4, 32, 6}) return launch_step_split<LAT, S, C, 4, 6>(inst, src, dst, a, configure_only);
+    if (r == ShapeRow{8, 32, 10}) return launch_step_mirror<LAT, S, C, 64, 10, false>(inst, src, dst, a, configure_only);
+    if (r == ShapeRow{8, 32, 12}) return launch_step_mirror<LAT, S, C, 64, 12, false>(inst, src, dst, a, configure_only);
+    if (r == ShapeRow{6, 128, 3}) return launch_step_t<LAT, S, C, 6, 128, 3>(inst, src, dst, a, configure_only);
   }
+  return cudaErrorInvalidConfiguration;  // no row is without a kernel
 }
 
 // ---------------------------------------------------------------------------
 // two steps in one launch
 // ---------------------------------------------------------------------------
-// Whether two steps per launch are the faster way.  Measured against the
-// share of pair_grid: 0.44 (384^2) 0.79 of the single step's speed, 0.57
-// (512^2) 1.03, 0.60 (100 x 6000) 1.18, 0.72 (768^2) 1.15, 0.80 (1024^2)
-// 1.19, 0.94 (4096^2) 1.25.
+// Whether steps go two per launch: shape index 0 leaves the choice open, and it
+// is the faster way.  Measured against the share of pair_grid: 0.44 (384^2)
+// 0.79 of the single step's speed, 0.57 (512^2) 1.03, 0.60 (100 x 6000) 1.18,
+// 0.72 (768^2) 1.15, 0.80 (1024^2) 1.19, 0.94 (4096^2) 1.25.
 template <int LAT, class S, class C>
 bool has_pair_t(const Instance* inst) {
   if constexpr (LAT == 0 && std::is_same<S, float>::value) {
-    return inst->pair.share >= 0.6;
+    return inst->shape.index == 0 && inst->pair.share >= 0.6;
   } else {
     return false;
   }

@@ -1,6 +1,7 @@
 // C ABI of the library (include/lbm.h): instance lifetime, validation,
 // device memory layout and the launch sequences of init / step / moments /
 // conservation sums.
+#include <algorithm>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -156,6 +157,10 @@ cudaError_t launch_conserve(const Instance* I, const void* src, double* partial,
   return launchers_of(I).conserve(I, src, partial, nblocks);
 }
 
+// Whether lbm_step takes two steps per launch (a graph of two steps is two
+// single ones: its launches swap the buffers an even number of times).
+bool steps_in_pairs(const Instance* I) { return I->graph_steps > 2 && launchers_of(I).has_pair(I); }
+
 // Enqueues the next step, or the next two in one launch where the instance
 // takes that way (pairs) and n >= 2, from buffer *cur; returns the steps
 // taken, or 0 with *e set.
@@ -268,7 +273,7 @@ cudaError_t capture_graph(Instance* I) {
   if (e == cudaSuccess) {
     // the launches swap the buffers an even number of times: the last two
     // steps of graph_steps = 4 m + 2 are single ones
-    const bool pairs = launchers_of(I).has_pair(I);
+    const bool pairs = steps_in_pairs(I);
     int c = I->cur, left = I->graph_steps;
     while (left > 0 && le == cudaSuccess)
       left -= advance_once(I, &c, left, pairs && (left > 2 || I->graph_steps % 4 == 0), &le);
@@ -429,7 +434,7 @@ int lbm_step(lbm_handle h, long n) {
       h->steps_done += h->graph_steps;
     }
   }
-  const bool pairs = h->graph_steps > 0 && n >= 2 && launchers_of(h).has_pair(h);
+  const bool pairs = n >= 2 && steps_in_pairs(h);
   while (n > 0) {
     cudaError_t e;
     const int k = advance_once(h, &h->cur, n, pairs, &e);
@@ -575,8 +580,8 @@ int lbm_shape_info(int lattice, int prec, int index, int* stage, int* block) {
   if (prec < kF64 || prec > kF32S16BF) return fail(LBM_EINVAL, "unknown precision");
   const Launchers& L = launchers_for(lattice, prec);
   if (index < 0 || index >= L.shape_count()) return fail(LBM_EINVAL, "shape index out of range");
-  int st = 0, bx = 0;
-  L.shape_get(index, &st, &bx);
+  int st = 0, bx = 0, minb = 0;
+  L.shape_get(nullptr, index, &st, &bx, &minb);
   if (stage) *stage = st;
   if (block) *block = bx;
   return LBM_OK;
@@ -590,6 +595,17 @@ int lbm_set_shape(lbm_handle h, int index) {
 }
 
 int lbm_get_shape(lbm_handle h) { return h ? h->shape.index : -1; }
+
+int lbm_step_info(lbm_handle h, int* stage, int* block, int* steps_per_launch) {
+  if (!h) return fail(LBM_EINVAL, "handle is NULL");
+  const bool pairs = steps_in_pairs(h);
+  int st = 0, bx = 0, minb = 0;
+  launchers_of(h).shape_get(h, h->shape.index, &st, &bx, &minb);
+  if (stage) *stage = pairs ? 10 : st;
+  if (block) *block = pairs ? kPairW : bx;
+  if (steps_per_launch) *steps_per_launch = pairs ? 2 : 1;
+  return LBM_OK;
+}
 
 int lbm_set_graph_steps(lbm_handle h, int steps) {
   if (!h) return fail(LBM_EINVAL, "handle is NULL");
@@ -620,15 +636,25 @@ int lbm_autotune(lbm_handle h, int reps, int* best_index, double* best_us) {
   const int keep = h->shape.index;
   int best = keep;
   float best_ms = 0.f;
+  int first[3], row[3];
+  launchers_of(h).shape_get(h, 0, first, first + 1, first + 2);
   for (int k = 0; k < n && e == cudaSuccess; ++k) {
     h->shape.index = k;
-    for (int w = 0; w < 2 && e == cudaSuccess; ++w) e = launch_step(h, h->buf[h->cur], h->buf[1 - h->cur]);
+    launchers_of(h).shape_get(h, k, row, row + 1, row + 2);
+    if (k > 0 && std::equal(row, row + 3, first)) continue;  // index 0's single step is this kernel
+    const bool pairs = steps_in_pairs(h);  // index 0 only
+    auto launch = [&]() {
+      return pairs ? launchers_of(h).step_pair(h, h->buf[h->cur], h->buf[1 - h->cur])
+                   : launch_step(h, h->buf[h->cur], h->buf[1 - h->cur]);
+    };
+    for (int w = 0; w < 2 && e == cudaSuccess; ++w) e = launch();
     if (e == cudaSuccess) e = cudaEventRecord(e0, h->stream);
-    for (int r = 0; r < reps && e == cudaSuccess; ++r) e = launch_step(h, h->buf[h->cur], h->buf[1 - h->cur]);
+    for (int r = 0; r < reps && e == cudaSuccess; ++r) e = launch();
     if (e == cudaSuccess) e = cudaEventRecord(e1, h->stream);
     if (e == cudaSuccess) e = cudaEventSynchronize(e1);
     float ms = 0.f;
     if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, e0, e1);
+    if (pairs) ms *= 0.5f;
     if (e == cudaSuccess && (k == 0 || ms < best_ms)) {
       best_ms = ms;
       best = k;

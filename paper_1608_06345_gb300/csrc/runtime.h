@@ -96,10 +96,11 @@ struct Launchers {
   int (*pool_grid)();
   int pool_tile_cells;  // cells per tile along x
   int (*shape_count)();
-  void (*shape_get)(int k, int* stage, int* bx);
+  // candidate k's single-step kernel, on inst (index 0 picks by its size) or, without one, on a large grid
+  void (*shape_get)(const Instance* inst, int k, int* stage, int* bx, int* minb);
   cudaError_t (*configure)(const Instance* inst);
   cudaError_t (*step_fd)(const Instance* inst, const void* src, void* dst, double lam);
-  bool (*has_pair)(const Instance* inst);  // whether two steps in one launch are the faster way here
+  bool (*has_pair)(const Instance* inst);  // whether steps go two per launch
   cudaError_t (*step_pair)(const Instance* inst, const void* src, void* dst);
 };
 

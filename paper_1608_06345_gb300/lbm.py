@@ -35,6 +35,7 @@ EXPORTS = ["lbm_state_bytes", "lbm_create", "lbm_destroy", "lbm_init", "lbm_init
            "lbm_conserved_noalloc", "lbm_pool_bytes", "lbm_pool_create", "lbm_pool_destroy",
            "lbm_pool_instance_bytes", "lbm_pool_submit", "lbm_pool_run", "lbm_pool_sync", "lbm_pool_poll",
            "lbm_pool_result", "lbm_pool_stats", "lbm_shape_info", "lbm_set_shape", "lbm_get_shape",
+           "lbm_step_info",
            "lbm_autotune", "lbm_set_graph_steps", "lbm_quadrature", "lbm_step_fd", "lbm_set_fd_kernel",
            "lbm_slab_plan",
            "lbm_slab_pack", "lbm_slab_unpack"]
@@ -111,6 +112,7 @@ def load(build_if_missing: bool = False):
         "lbm_shape_info": (ctypes.c_int, [ctypes.c_int, ctypes.c_int, ctypes.c_int, ip, ip]),
         "lbm_set_shape": (ctypes.c_int, [vp, ctypes.c_int]),
         "lbm_get_shape": (ctypes.c_int, [vp]),
+        "lbm_step_info": (ctypes.c_int, [vp, ip, ip, ip]),
         "lbm_autotune": (ctypes.c_int, [vp, ctypes.c_int, ip, dp]),
         "lbm_set_graph_steps": (ctypes.c_int, [vp, ctypes.c_int]),
         "lbm_set_fd_kernel": (ctypes.c_int, [vp, ctypes.c_int]),
@@ -266,6 +268,13 @@ def lbm_set_shape(h, index):
 
 def lbm_get_shape(h):
     return load().lbm_get_shape(h)
+
+
+def lbm_step_info(h):
+    """(stage, block, steps per launch) of what lbm_step launches."""
+    st, bx, n = ctypes.c_int(), ctypes.c_int(), ctypes.c_int()
+    _check(load().lbm_step_info(h, ctypes.byref(st), ctypes.byref(bx), ctypes.byref(n)))
+    return st.value, bx.value, n.value
 
 
 def lbm_quadrature(reps, exps, r0=1.0):
