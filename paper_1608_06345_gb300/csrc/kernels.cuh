@@ -242,20 +242,9 @@ __device__ __forceinline__ unsigned ld_again(const unsigned* p) {
   return v;
 }
 
-__device__ __forceinline__ float2 ld_again(const float2* p) {
-  float2 v;
-  asm volatile("ld.global.nc.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p));
-  return v;
-}
-__device__ __forceinline__ uint2 ld_again(const uint2* p) {
-  uint2 v;
-  asm volatile("ld.global.nc.v2.b32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "l"(p));
-  return v;
-}
-
 // ---------------------------------------------------------------------------
-// two FP32 values in one 64-bit register; add, multiply and fma work on both
-// in one instruction, each rounded as the scalar one is
+// two FP32 values in one 64-bit register; add and subtract work on both in one
+// instruction, each rounded as the scalar one is
 // ---------------------------------------------------------------------------
 using f32x2 = unsigned long long;
 __device__ __forceinline__ f32x2 pack_f32x2(float a, float b) {
@@ -263,7 +252,6 @@ __device__ __forceinline__ f32x2 pack_f32x2(float a, float b) {
   asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "f"(a), "f"(b));
   return v;
 }
-__device__ __forceinline__ f32x2 both(float a) { return pack_f32x2(a, a); }
 __device__ __forceinline__ void unpack_f32x2(f32x2 v, float& a, float& b) {
   asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
 }
@@ -278,16 +266,6 @@ __device__ __forceinline__ f32x2 sub_f32x2(f32x2 a, f32x2 b) {
   return v;
 }
 __device__ __forceinline__ f32x2 neg_f32x2(f32x2 a) { return a ^ 0x8000000080000000ull; }
-__device__ __forceinline__ f32x2 mul_f32x2(f32x2 a, f32x2 b) {
-  f32x2 v;
-  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(v) : "l"(a), "l"(b));
-  return v;
-}
-__device__ __forceinline__ f32x2 fma_f32x2(f32x2 a, f32x2 b, f32x2 c) {
-  f32x2 v;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(v) : "l"(a), "l"(b), "l"(c));
-  return v;
-}
 
 // ---------------------------------------------------------------------------
 // equilibrium deviations (Eq. (18), regrouped by powers of s per group)
