@@ -412,11 +412,11 @@ cudaError_t launch_step_fd_t(const Instance* inst, const void* src, void* dst, d
   };
   if constexpr (LAT == 0) {
     if constexpr (IsS16<S>::value)
-      if (tiles(32, 8, 1) >= 3 * 152) return launch_step_fd_tile<LAT, S, C, 32, 8, 1, 3>(inst, src, dst, lam);
+      if (tiles(32, 8, 1) >= 3 * device_sms()) return launch_step_fd_tile<LAT, S, C, 32, 8, 1, 3>(inst, src, dst, lam);
     return launch_step_fd_row<LAT, S, C, 128>(inst, src, dst, lam);
   } else {
     if constexpr (sizeof(S) == 8) {
-      if (tiles(16, 4, 4) >= 2 * 152) return launch_step_fd_tile<LAT, S, C, 16, 4, 4, 2>(inst, src, dst, lam);
+      if (tiles(16, 4, 4) >= 2 * device_sms()) return launch_step_fd_tile<LAT, S, C, 16, 4, 4, 2>(inst, src, dst, lam);
     } else {
       if (tiles(16, 8, 4) >= 64) return launch_step_fd_tile<LAT, S, C, 16, 8, 4, 2>(inst, src, dst, lam);
     }
