@@ -45,7 +45,7 @@ enum lbm_status {
   LBM_ECUDA = 3,      /* a CUDA runtime call failed */
   LBM_ENONFINITE = 4, /* a step produced a non-finite density or temperature */
   LBM_ETIMEOUT = 5,   /* a bounded wait inside the two-step kernel (lbm_step) gave
-                         up after about a second: the state is not valid */
+                         up (lbm_set_wait_limit): the state is not valid */
   LBM_EBUSY = 6       /* a pool's memory budget is full */
 };
 
@@ -132,6 +132,12 @@ int lbm_step(lbm_handle h, long n);
  * step separately (the plain one-launch-per-step path, whatever the shape).  Execution control
  * with no counterpart in the paper. */
 int lbm_set_graph_steps(lbm_handle h, int steps);
+
+/* Tries, of about a microsecond each, after which a wait of the two-step
+ * kernel's warps for one another gives up and the run ends in LBM_ETIMEOUT
+ * (default 2^20, a second; 0: at once, whether or not there is anything to
+ * wait for).  Execution control with no counterpart in the paper. */
+int lbm_set_wait_limit(lbm_handle h, int tries);
 
 /* Advance n >= 0 time steps of the finite-difference variant of Sec. III:
  * forward Euler in time, the convection xi_i . grad q_i discretised along

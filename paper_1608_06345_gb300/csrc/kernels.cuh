@@ -1488,8 +1488,8 @@ __device__ __forceinline__ int map_coord(int q, int n, int bc) {
 }
 
 // mbarriers of the ring (one arrival per warp of a group); a wait gives up
-// after about a second, so that no fault elsewhere can leave a block spinning
-constexpr int kWaitTries = 1 << 20;
+// after a number of tries of about a microsecond each, so that no fault
+// elsewhere can leave a block spinning (lbm_set_wait_limit)
 
 __device__ __forceinline__ void bar_init(unsigned long long* b, unsigned count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"((unsigned)__cvta_generic_to_shared(b)), "r"(count));
@@ -1497,10 +1497,10 @@ __device__ __forceinline__ void bar_init(unsigned long long* b, unsigned count) 
 __device__ __forceinline__ void bar_arrive(unsigned long long* b) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"((unsigned)__cvta_generic_to_shared(b)) : "memory");
 }
-__device__ __forceinline__ bool bar_wait(unsigned long long* b, unsigned parity) {
+__device__ __forceinline__ bool bar_wait(unsigned long long* b, unsigned parity, int tries) {
   const unsigned at = (unsigned)__cvta_generic_to_shared(b);
   unsigned done = 0;
-  for (int n = 0; n < kWaitTries && !done; ++n)
+  for (int n = 0; n < tries && !done; ++n)
     asm volatile(
         "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, 1000;\n selp.u32 %0, 1, 0, p;\n}"
         : "=r"(done)
@@ -1511,7 +1511,7 @@ __device__ __forceinline__ bool bar_wait(unsigned long long* b, unsigned parity)
 
 template <bool IDX32>
 __global__ void __launch_bounds__(4 * kPairW, 1) k_step_pair(const float* __restrict__ src, float* __restrict__ dst,
-                                                             const Args<float> a, int w) {
+                                                             const Args<float> a, int w, int tries) {
   using L = Lat<0>;
   using S = float;
   using C = float;
@@ -1536,7 +1536,7 @@ __global__ void __launch_bounds__(4 * kPairW, 1) k_step_pair(const float* __rest
     if ((threadIdx.x & 31) == 0) bar_arrive(b);
   };
   auto wait = [&](unsigned long long* b, int n) {  // for row n's arrivals
-    const bool ok = bar_wait(b + (n & (NB - 1)), (n / NB) & 1);
+    const bool ok = bar_wait(b + (n & (NB - 1)), (n / NB) & 1, tries);
     if (!ok) atomicOr(a.flag, 2u);
     return ok;
   };

@@ -347,7 +347,7 @@ cudaError_t launch_pair_v(const Instance* inst, const void* src, void* dst, bool
   if (configure_only) return cudaSuccess;
   const PairGrid& g = inst->pair;
   return launch_next(kern, dim3((unsigned)g.strips, (unsigned)g.bands), 4 * kPairW, smem, inst->stream,
-                     static_cast<const float*>(src), static_cast<float*>(dst), inst->af, g.width);
+                     static_cast<const float*>(src), static_cast<float*>(dst), inst->af, g.width, inst->wait_tries);
 }
 
 template <int LAT, class S, class C>

@@ -227,6 +227,7 @@ int prepare_instance(Instance* I, int lattice, double gamma, double tau_f, doubl
   I->shape = default_shape(lattice, grid->prec);
   I->fd_kernel = LBM_FD_AUTO;
   I->graph_steps = 64;
+  I->wait_tries = kPairTries;
   I->graph_shape = -1;
   I->graph_exec = nullptr;
   I->graph = nullptr;
@@ -614,6 +615,17 @@ int lbm_set_graph_steps(lbm_handle h, int steps) {
     cudaStreamSynchronize(h->stream);
     drop_graph(h);
     h->graph_steps = steps;
+  }
+  return LBM_OK;
+}
+
+int lbm_set_wait_limit(lbm_handle h, int tries) {
+  if (!h) return fail(LBM_EINVAL, "handle is NULL");
+  if (tries < 0) return fail(LBM_EINVAL, "tries must be >= 0");
+  if (tries != h->wait_tries) {
+    cudaStreamSynchronize(h->stream);
+    drop_graph(h);
+    h->wait_tries = tries;
   }
   return LBM_OK;
 }

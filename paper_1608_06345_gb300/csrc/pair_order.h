@@ -42,6 +42,7 @@ constexpr int pair_a_stored(int t) { return t < kPairBars ? t - 3 : -1; }
 constexpr int pair_b_begin(int q) { return q + 5; }
 constexpr int pair_b_end(int q) { return q + 6; }
 
+constexpr int kPairTries = 1 << 20;   // of a wait, about a microsecond each
 constexpr int kPairW = 128;           // A's columns
 constexpr int kPairOut = kPairW - 6;  // columns a strip can hold
 

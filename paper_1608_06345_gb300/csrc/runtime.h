@@ -52,7 +52,8 @@ struct Instance {
   int graph_shape;           // shape index the graph was captured with
   cudaGraphExec_t graph_exec;
   cudaGraph_t graph;
-  PairGrid pair;  // of a D2Q37 FP32 instance (lbm_create)
+  PairGrid pair;   // of a D2Q37 FP32 instance (lbm_create)
+  int wait_tries;  // of a wait inside the two-step kernel
 };
 
 // Bytes of the tail region after the two buffers.

@@ -35,7 +35,7 @@ EXPORTS = ["lbm_state_bytes", "lbm_create", "lbm_destroy", "lbm_init", "lbm_init
            "lbm_conserved_noalloc", "lbm_pool_bytes", "lbm_pool_create", "lbm_pool_destroy",
            "lbm_pool_instance_bytes", "lbm_pool_submit", "lbm_pool_run", "lbm_pool_sync", "lbm_pool_poll",
            "lbm_pool_result", "lbm_pool_stats", "lbm_shape_info", "lbm_set_shape", "lbm_get_shape",
-           "lbm_step_info",
+           "lbm_step_info", "lbm_set_wait_limit",
            "lbm_autotune", "lbm_set_graph_steps", "lbm_quadrature", "lbm_step_fd", "lbm_set_fd_kernel",
            "lbm_slab_plan",
            "lbm_slab_pack", "lbm_slab_unpack"]
@@ -115,6 +115,7 @@ def load(build_if_missing: bool = False):
         "lbm_step_info": (ctypes.c_int, [vp, ip, ip, ip]),
         "lbm_autotune": (ctypes.c_int, [vp, ctypes.c_int, ip, dp]),
         "lbm_set_graph_steps": (ctypes.c_int, [vp, ctypes.c_int]),
+        "lbm_set_wait_limit": (ctypes.c_int, [vp, ctypes.c_int]),
         "lbm_set_fd_kernel": (ctypes.c_int, [vp, ctypes.c_int]),
         "lbm_quadrature": (ctypes.c_int, [ctypes.c_int, ctypes.c_int, ip, ctypes.c_int, ip, ctypes.c_double, ip,
                                           dp, dp, dp]),
@@ -295,6 +296,10 @@ def lbm_quadrature(reps, exps, r0=1.0):
 
 def lbm_set_graph_steps(h, steps):
     return _check(load().lbm_set_graph_steps(h, int(steps)))
+
+
+def lbm_set_wait_limit(h, tries):
+    return _check(load().lbm_set_wait_limit(h, int(tries)))
 
 
 def lbm_set_fd_kernel(h, kernel):
