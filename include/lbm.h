@@ -268,7 +268,7 @@ int lbm_get_shape(lbm_handle h);
  * Any pointer may be NULL. */
 int lbm_step_info(lbm_handle h, int* stage, int* block, int* steps_per_launch);
 
-/* Time every candidate shape on this instance's own buffers (reps launches
+/* Time every candidate shape on this instance's own buffers (reps steps
  * each, CUDA events on its stream; the trials write only the idle buffer,
  * so the state does not change), select the fastest and return its index
  * and mean time per step in microseconds.  Index 0 is timed as lbm_step runs

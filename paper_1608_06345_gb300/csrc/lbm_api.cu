@@ -659,14 +659,15 @@ int lbm_autotune(lbm_handle h, int reps, int* best_index, double* best_us) {
       return pairs ? launchers_of(h).step_pair(h, h->buf[h->cur], h->buf[1 - h->cur])
                    : launch_step(h, h->buf[h->cur], h->buf[1 - h->cur]);
     };
-    for (int w = 0; w < 2 && e == cudaSuccess; ++w) e = launch();
+    const int launches = pairs ? (reps + 1) / 2 : reps;
+    for (int w = pairs ? 1 : 0; w < 2 && e == cudaSuccess; ++w) e = launch();
     if (e == cudaSuccess) e = cudaEventRecord(e0, h->stream);
-    for (int r = 0; r < reps && e == cudaSuccess; ++r) e = launch();
+    for (int r = 0; r < launches && e == cudaSuccess; ++r) e = launch();
     if (e == cudaSuccess) e = cudaEventRecord(e1, h->stream);
     if (e == cudaSuccess) e = cudaEventSynchronize(e1);
     float ms = 0.f;
     if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, e0, e1);
-    if (pairs) ms *= 0.5f;
+    ms /= (float)(pairs ? 2 * launches : launches);
     if (e == cudaSuccess && (k == 0 || ms < best_ms)) {
       best_ms = ms;
       best = k;
@@ -680,7 +681,7 @@ int lbm_autotune(lbm_handle h, int reps, int* best_index, double* best_us) {
   }
   h->shape.index = best;
   if (best_index) *best_index = best;
-  if (best_us) *best_us = 1e3 * best_ms / reps;
+  if (best_us) *best_us = 1e3 * best_ms;
   return LBM_OK;
 }
 
