@@ -399,26 +399,46 @@ cudaError_t launch_step_fd_row(const Instance* inst, const void* src, void* dst,
 }
 
 // The faster of the two per lattice, storage and size (large grids: figures at
-// k_step_fd_tile).  A tile's block is long and large, so grids of few tiles
-// leave SMs idle that the row kernel's smaller blocks would use; us per step,
-// tile and row: D3Q107 FP32 32^3 (64 tiles) 74 / 72, 40^3 (150) 97 / 127, 1000
-// x 4 x 4 (63) 59 / 37; FP16 storage 32^3 57 / 63; FP64 32^3 (128) 553 / 380,
-// 48^3 (432) 878 / 1238; D2Q37 FP16 storage 256^2 (256) 13.1 / 11.1, 512^2
+// k_step_fd_tile).  us per step, tile / row.
+//   A tile's block is long and large, so grids of few tiles leave SMs idle that
+// the row kernel's smaller blocks would use: D3Q107 FP32 64 x 64 x 6 (24576
+// cells) 60 / 36, 40 x 100 x 5 (20000) 59 / 36, 1000 x 4 x 4 (16000) 59 / 37,
+// 32^3 (32768) 74 / 72, 2000 x 4 x 4 (32000) 54 / 57, 40^3 88 / 137; FP16
+// storage 40 x 100 x 5 45 / 31, 32^3 57 / 63; FP64 32^3 (128 tiles) 553 / 380,
+// 48^3 (432) 878 / 1238; D2Q37 FP16 storage 256^2 (256 tiles) 13.1 / 11.1, 512^2
 // (1024) 27.1 / 29.6.
+//   Nor does it pay where the grid is so thin along y or z that its tiles hold
+// more threads without a cell than the row kernel's blocks, by a factor that
+// depends on the tile's gain on full ones: D3Q107 FP32 2.8 (1000 x 9 x 5) 80 /
+// 113, 3.5 (4000 x 3 x 3) 66 / 59, 3.8 (300 x 300 x 1) 230 / 168, 32 (20000 x 1 x
+// 1) 194 / 34; FP16 storage 1.28 (300 x 300 x 3) 308 / 345, 1.31 (1000 x 40 x
+// 3) 187 / 138, 1.5 (300 x 5 x 300) 518 / 448, 32 (20000 x 1 x 1) 171 / 28; D2Q37 FP16 storage
+// 2 (100000 x 4) 46 / 53, 4 (100000 x 2) 31 / 24, 8 (100000 x 1) 26 / 13.  FP64 is
+// bound by the FP64 pipe, whose time is that of the warps with a cell (16 x 2 of
+// a tile, 32 of a row): 1.06 times as many (300 x 9 x 300) 6740 / 7189, 1.09 (1000
+// x 9 x 5) 561 / 619, 1.27 (300 x 3 x 300) 2797 / 2412, 2 (20000 x 1 x 1) 563 / 219.
 template <int LAT, class S, class C>
 cudaError_t launch_step_fd_t(const Instance* inst, const void* src, void* dst, double lam) {
-  auto tiles = [&](int bx, int by, int bz) {
-    return ((long long)inst->n[0] + bx - 1) / bx * ((inst->n[1] + by - 1) / by) * ((inst->n[2] + bz - 1) / bz);
+  auto blocks = [&](long long bx, int by, int bz) {
+    return (inst->n[0] + bx - 1) / bx * ((inst->n[1] + by - 1) / by) * ((inst->n[2] + bz - 1) / bz);
   };
   if constexpr (LAT == 0) {
-    if constexpr (IsS16<S>::value)
-      if (tiles(32, 8, 1) >= 3 * device_sms()) return launch_step_fd_tile<LAT, S, C, 32, 8, 1, 3>(inst, src, dst, lam);
+    if constexpr (IsS16<S>::value) {
+      const long long tiles = blocks(32, 8, 1);
+      if (tiles >= 3 * device_sms() && tiles * 256 <= 2 * 128 * blocks(128, 1, 1))
+        return launch_step_fd_tile<LAT, S, C, 32, 8, 1, 3>(inst, src, dst, lam);
+    }
     return launch_step_fd_row<LAT, S, C, 128>(inst, src, dst, lam);
   } else {
     if constexpr (sizeof(S) == 8) {
-      if (tiles(16, 4, 4) >= 2 * device_sms()) return launch_step_fd_tile<LAT, S, C, 16, 4, 4, 2>(inst, src, dst, lam);
+      const long long tiles = blocks(16, 4, 4);
+      if (tiles >= 2 * device_sms() && 10 * blocks(16, 2, 1) <= 11 * blocks(32, 1, 1) &&
+          2 * tiles * 256 <= 5 * 64 * blocks(64, 1, 1))
+        return launch_step_fd_tile<LAT, S, C, 16, 4, 4, 2>(inst, src, dst, lam);
     } else {
-      if (tiles(16, 8, 4) >= 64) return launch_step_fd_tile<LAT, S, C, 16, 8, 4, 2>(inst, src, dst, lam);
+      const long long tiles = blocks(16, 8, 4), row = 64 * blocks(64, 1, 1);
+      if (inst->N >= 200LL * device_sms() && 10 * tiles * 512 <= (IsS16<S>::value ? 13 : 30) * row)
+        return launch_step_fd_tile<LAT, S, C, 16, 8, 4, 2>(inst, src, dst, lam);
     }
     return launch_step_fd_row<LAT, S, C, 64>(inst, src, dst, lam);
   }

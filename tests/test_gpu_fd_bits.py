@@ -14,9 +14,9 @@ CASES = [
     # lattice, prec, small grid, boundaries, copies (tiles of the small and the repeated grid; the line lies at)
     (1, 0, (33, 20, 20), (1, 0, 0), 5),  # 75 and 375 tiles of 16 x 4 x 4 (two per SM)
     (1, 0, (33, 21, 19), (0, 1, 0), 6),  # ragged in y and z: 90 and 522
-    (1, 1, (33, 20, 6), (0, 1, 0), 6),   # 18 and 81 of 16 x 8 x 4 (64)
-    (1, 2, (33, 20, 6), (1, 0, 0), 6),
-    (1, 3, (20, 17, 7), (1, 1, 0), 7),   # 12 and 78
+    (1, 1, (33, 20, 6), (0, 1, 0), 10),  # 3960 and 39600 cells (200 per SM)
+    (1, 2, (33, 20, 6), (1, 0, 0), 10),
+    (1, 3, (20, 17, 7), (1, 1, 0), 14),  # 2380 and 33320
     (0, 2, (100, 40), (1, 0), 30),       # 20 and 600 of 32 x 8 (three per SM)
     (0, 3, (75, 41), (0, 0), 40),        # 18 and 615
 ]
