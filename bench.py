@@ -143,7 +143,7 @@ def measured_peaks():
 
 
 # the sources that define each recorded kernel (its code and launch shapes)
-KERNEL_SOURCES = {"k_step": ("kernels.cuh", "launch_impl.cuh"),
+KERNEL_SOURCES = {"k_step": ("kernels.cuh", "launch_impl.cuh", "pair_order.h"),
                   "k_step_fd": ("kernels.cuh", "launch_impl.cuh", "fd_march.cuh")}
 
 
