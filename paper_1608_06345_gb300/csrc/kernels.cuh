@@ -1713,7 +1713,7 @@ __global__ void __launch_bounds__(BX) k_step_fd(const S* __restrict__ src, S* __
 // 112 x 96 x 80 FP32 2069 -> 800, FP16 storage 940 -> 731; 256 x 128 x 128
 // 9879 -> 3820 and 5543 -> 3488.  D2Q37 FP16 storage 4096^2 1789 -> 1537,
 // FP32 2613 -> 2690, which keeps k_step_fd; D3Q107 FP64 256 x 128 x 128 33.8
-// -> 31.2 ms.  Also tried: tiles of 32 x 4 x 4 and 32 x 2 x 4, 0 to 10% more;
+// -> 30.2 ms.  Also tried: tiles of 32 x 4 x 4 and 32 x 2 x 4, 0 to 10% more;
 // the second pass as a loop over the pairs with the next direction's loads
 // ahead, 883 (112 x 96 x 80 FP32); that in f32x2 arithmetic, two cells per
 // thread, 693, but with other roundings.
@@ -1934,7 +1934,9 @@ __global__ void k_moments(const S* __restrict__ src, double* __restrict__ rho, d
 // 127 353 -> 377, FP16 storage 379 -> 336; D2Q37 FP32 300^2 20.6 -> 24.1 (four
 // cells per thread carry all 34 FP64 additions).  Without the next group's
 // first loads issued before the present group's FP64 additions 261, 218, 398,
-// 370 us; runs of 16 cells 232, 199, 378, 341.
+// 370 us; runs of 16 cells 232, 199, 378, 341.  lbm_conserved_noalloc, 16
+// cells per thread, the whole call: 296 -> 246, 200 -> 221, 397 -> 370, 503 ->
+// 345.
 // ---------------------------------------------------------------------------
 constexpr int kRedMaxBlocks = 1024;  // partials an instance has room for
 constexpr int kRedVals = 5;  // mass, momentum[3], energy
